@@ -1,11 +1,10 @@
 // batched.cu -- many independent assignment problems in one persistent launch.
 //
 // Each CTA pulls problems from a queue in longest-first order (LPT on n) and
-// runs the whole main routine of Sec. 2.2 on one problem with every piece of
-// per-problem state in shared memory: the keys k(A), the proposal words, the
-// row duals, the free-row lists and the proposal lists.  Rounds are separated
-// by __syncthreads() instead of a grid barrier.  Only the rounded cost rows
-// are read from global memory (HBM / L2), one warp per row.
+// runs the whole main routine of Sec. 2.2 on one problem (cta_solve.cuh) with
+// every piece of per-problem state in shared memory.  Rounds are separated by
+// __syncthreads() instead of a grid barrier.  Only the rounded cost rows are
+// read from global memory (HBM / L2).
 //
 // Problem i is square (n_i rows and columns).  Packed layouts:
 //   costs   C[c_off_i + b * n_i + a], c_off_i = sum_{j<i} n_j^2 (rows = B)
@@ -25,14 +24,14 @@
 #include "scan_common.cuh"
 #include "quantise.cuh"
 #include "points.cuh"
+#include "cta_solve.cuh"
 
 namespace prot {
 namespace {
 
 constexpr int kMaxN = 5000;               // largest problem whose state fits shared memory
-constexpr int kRowBits = 13;              // a free-list entry: row | resume column << 13
-constexpr int kRowMask = (1 << kRowBits) - 1;
-static_assert(kMaxN < (1 << kRowBits), "rows and resume columns must fit 13 bits");
+static_assert(kMaxN <= kCtaMaxCols, "rows and resume columns must fit the CTA solver's list entries");
+constexpr int kCostSums = 256;            // partial sums of a problem's cost at the default launch shape
 constexpr int kMaxCbarByte = 252;         // byte storage when floor(1/eps) <= 252 (as pr_assign)
 
 struct BDesc {
@@ -79,7 +78,7 @@ struct BParams {
     const void *cb;  // uint8_t or uint16_t, as k_bsolve is instantiated
     int nprob;
     int n_max;
-    int ldq_max;
+    int cost_sums;  // strided partial sums of a problem's cost
     // cost source for the reported costs
     const void *C;
     int dt;  // PR_F32 / PR_F64 (matrix source)
@@ -284,318 +283,72 @@ __global__ void k_bpoints_quant(const float *__restrict__ XA, const float *__res
 // ---------------------------------------------------------------------------
 // The per-problem solver.
 // ---------------------------------------------------------------------------
-struct BShared {
-    int nfl[2], nql[2], nwon;
-    int had_prop, nonfirst;
-    int cur_problem;
-    int total;
-    int warp_tot[32];
-    unsigned long long bytes, rows;
+// The reported cost of a matched pair of one problem: the input matrix's
+// entry, or the FP64 distance of the matched points (input units).
+struct BatchCost {
+    const BParams &p;
+    const BDesc &D;
+    __device__ double operator()(int b, int a) const {
+        if (p.points)
+            return dist_f64(p.XB + (long long)(D.v_off + b) * p.dim, p.XA + (long long)(D.v_off + a) * p.dim, p.dim,
+                            p.squared);
+        const long long at = D.c_off + (long long)b * D.n + a;
+        return p.dt == PR_F64 ? reinterpret_cast<const double *>(p.C)[at]
+                              : (double)reinterpret_cast<const float *>(p.C)[at];
+    }
 };
-
-// Lowest column a >= start of the row with cbar + k(a) == tgt whose word does
-// not carry a tag in [Rps, R) (taken earlier in this phase), or -1.  UNROLL
-// 16-byte loads per lane are in flight per step.
-template <int UNROLL, class CB, bool F7>
-__device__ __forceinline__ int warp_scan_row(const CB *__restrict__ row, const CB *ks,
-                                             const unsigned long long *pw, int start, int ldq,
-                                             uint32_t tgt, unsigned R, unsigned Rps, int lane,
-                                             unsigned long long &bytes) {
-    constexpr int W = 16 / (int)sizeof(CB);  // columns per 16-byte load
-    constexpr unsigned kAll = W == 16 ? 0xFFFFu : 0xFFu;
-    const uint32_t t2 = W == 8 ? (tgt | (tgt << 16)) : tgt * 0x01010101u;
-    const bool check_taken = R > Rps;
-    for (int c0 = start & ~(W - 1); c0 < ldq; c0 += 32 * W * UNROLL) {
-        uint4 cv[UNROLL];
-#pragma unroll
-        for (int u = 0; u < UNROLL; ++u) {
-            const int idx = c0 + u * 32 * W + lane * W;
-            cv[u] = idx < ldq ? ld_nc_na_v4(row + idx) : make_uint4(0, 0, 0, 0);
-        }
-        bytes += sizeof(CB) * (unsigned long long)min(32 * W * UNROLL, ldq - c0);
-#pragma unroll
-        for (int u = 0; u < UNROLL; ++u) {
-            const int idx = c0 + u * 32 * W + lane * W;
-            unsigned m = 0;
-            if (idx < ldq) {
-                const uint4 kv = *reinterpret_cast<const uint4 *>(ks + idx);
-                m = W == 8 ? eq_mask(make_uint4(cv[u].x + kv.x, cv[u].y + kv.y, cv[u].z + kv.z, cv[u].w + kv.w), t2)
-                           : eq_mask8<F7>(cv[u], kv, t2);
-            }
-            const int lo = start - idx;
-            if (lo > 0) m &= lo >= W ? 0u : (kAll << lo) & kAll;
-            for (;;) {
-                const unsigned any = __ballot_sync(0xFFFFFFFFu, m != 0);
-                if (any == 0) break;
-                const int L = __ffs(any) - 1;
-                const int a = __shfl_sync(0xFFFFFFFFu, idx + __ffs(m) - 1, L);
-                bool taken = false;
-                if (check_taken) {
-                    const unsigned t = tag_of(pw[a]);
-                    taken = t >= Rps && t < R;
-                }
-                if (!taken) return a;
-                if (lane == L) m &= m - 1;
-            }
-        }
-    }
-    return -1;
-}
-
-__device__ __forceinline__ int block_scan_excl(int flag, BShared &s) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const unsigned bal = __ballot_sync(0xFFFFFFFFu, flag);
-    const int within = __popc(bal & ((1u << lane) - 1));
-    if (lane == 0) s.warp_tot[warp] = __popc(bal);
-    __syncthreads();
-    if (warp == 0) {
-        const int v = lane < nw ? s.warp_tot[lane] : 0;
-        int x = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane < nw) s.warp_tot[lane] = x - v;
-        if (lane == 31) s.total = x;
-    }
-    __syncthreads();
-    const int r = s.warp_tot[warp] + within;
-    __syncthreads();
-    return r;
-}
 
 // F7: floor(1/eps) <= 125, so every sum of a real column's cbar and key
 // stays below 256 and the byte pre-test is one plain add (may_match<true>).
 template <int THREADS, int UNROLL, class CB, bool F7>
 __global__ void __launch_bounds__(THREADS, 1) k_bsolve(BParams p) {
     extern __shared__ __align__(16) unsigned char dyn[];
-    __shared__ BShared s;
-    // region sizes use n_max rounded up to a multiple of 8, so every region
-    // (8-byte words, int2 pairs, the uint4-read key copy) starts 16-byte aligned
-    const int nmax = (p.n_max + 7) & ~7;
-    unsigned long long *pw = reinterpret_cast<unsigned long long *>(dyn);
-    int *yb = reinterpret_cast<int *>(pw + nmax);
-    int *fl0 = yb + nmax;
-    int *fl1 = fl0 + nmax;
-    int2 *ql0 = reinterpret_cast<int2 *>(fl1 + nmax);
-    int2 *ql1 = ql0 + nmax;
-    int *won = reinterpret_cast<int *>(ql1 + nmax);
-    CB *ks = reinterpret_cast<CB *>(won + nmax);  // keys in the stored type (bytes: padding 0xFF)
-    int *fl[2] = {fl0, fl1};
-    int2 *ql[2] = {ql0, ql1};
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-    if (threadIdx.x == 0) s.bytes = s.rows = 0;
+    __shared__ CtaShared s;
+    __shared__ int cur_problem;
+    __shared__ double part[THREADS > kCostSums ? THREADS : kCostSums];
+    const CtaLayout L(p.n_max, p.n_max);
+    const CtaState<CB> state(dyn, L);
     long long my_phases = 0, my_rounds = 0;
+    unsigned long long my_bytes = 0, my_rows = 0;  // thread 0's
 
     for (;;) {
         if (threadIdx.x == 0) {
             int t = (int)atomicAdd(&p.ctl->queue, 1u);
             if (ld_relaxed_s32(&p.ctl->head.abort)) t = p.nprob;  // stop after an error
-            s.cur_problem = t;
+            cur_problem = t;
         }
         __syncthreads();
-        const int t = s.cur_problem;
+        const int t = cur_problem;
         __syncthreads();  // every thread has read cur_problem before it changes
         if (t >= p.nprob) break;
         const int pi = p.order[t];
         const BDesc D = p.desc[pi];
-        const int n = D.n, ldq = D.ldq;
         const CB *cb = static_cast<const CB *>(p.cb) + D.cb_off;
-
-        // Initialisation (Sec. 2.2): y(b) = eps, y(a) = 0, M empty, B' = B.
-        for (int a = threadIdx.x; a < ldq; a += blockDim.x) ks[a] = a < n ? (CB)0 : (CB)(sizeof(CB) == 1 ? 0xFF : kPadKey);
-        for (int a = threadIdx.x; a < n; a += blockDim.x) pw[a] = word_of(0, -1);
-        for (int b = threadIdx.x; b < n; b += blockDim.x) {
-            yb[b] = 1;
-            fl0[b] = b;
-        }
+        CtaCounts c = {0, 0, 0, 0, false};
+        cta_init(s, state, D.n, D.n, D.ldq);
+        cta_phases<UNROLL, CB, F7, false>(s, state, cb, D.n, D.n, D.ldq, D.T, D.cap, 0u, D.n, c);
+        my_phases += c.phases;
+        my_rounds += c.rounds;
         if (threadIdx.x == 0) {
-            s.nfl[0] = n;
-            s.nfl[1] = 0;
+            my_bytes += s.bytes;
+            my_rows += s.rows;
         }
-        __syncthreads();
-
-        unsigned R = 0;
-        long long phases = 0;
-        int cur = 0, qcur = 0;
-        bool failed = false;
-        for (;;) {
-            const int nf = s.nfl[cur];
-            if (nf <= D.T) break;
-            if (phases >= D.cap) {
-                failed = true;
-                break;
-            }
-            ++phases;
-            const unsigned Rps = R + 1;
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                s.nfl[cur ^ 1] = 0;
-                s.nwon = 0;
-            }
-            bool first = true;
-            for (;;) {
-                ++R;
-                if (threadIdx.x == 0) {
-                    s.nql[qcur] = 0;
-                    s.had_prop = 0;
-                    s.nonfirst = 0;
-                }
-                __syncthreads();
-                const int items = first ? nf : s.nql[qcur ^ 1];
-                unsigned long long my_bytes = 0;
-                for (int it = warp; it < items; it += nwarps) {
-                    int b, start = 0;
-                    if (first) {
-                        // b, or b | (resume column << 13) for an evicted row
-                        const int e = fl[cur][it];
-                        b = e & kRowMask;
-                        start = e >> kRowBits;
-                    } else {
-                        const int2 q = ql[qcur ^ 1][it];
-                        b = q.x;
-                        if (row_of(pw[q.y]) == b) continue;  // won: matched
-                        start = q.y + 1;                     // lost: resume after a
-                    }
-                    const uint32_t tgt = (uint32_t)(yb[b] - 1);
-                    const int a = warp_scan_row<UNROLL, CB, F7>(cb + (long long)b * ldq, ks, pw, start, ldq, tgt, R,
-                                                            Rps, lane, my_bytes);
-                    if (lane == 0) {
-                        if (a >= 0) {
-                            const unsigned long long old = atomicMax(pw + a, word_of(R, b));
-                            if (tag_of(old) < Rps) {
-                                // first proposal: a is won this round (step III a
-                                // at the phase end), its partner is evicted (II)
-                                won[atomicAdd(&s.nwon, 1)] = a;
-                                // the evicted row resumes after a: every column
-                                // <= a is above its (unchanged) target for good
-                                const int partner = row_of(old);
-                                if (partner >= 0)
-                                    fl[cur ^ 1][atomicAdd(&s.nfl[cur ^ 1], 1)] = partner | ((a + 1) << kRowBits);
-                            } else {
-                                s.nonfirst = 1;
-                            }
-                            const int j = atomicAdd(&s.nql[qcur], 1);
-                            ql[qcur][j] = make_int2(b, a);
-                            s.had_prop = 1;
-                        } else {
-                            yb[b] += 1;  // step (III b): relabel
-                            fl[cur ^ 1][atomicAdd(&s.nfl[cur ^ 1], 1)] = b;
-                        }
-                    }
-                }
-                if (lane == 0) {
-                    if (my_bytes) atomicAdd(&s.bytes, my_bytes);
-                }
-                __syncthreads();
-                const bool had = s.had_prop != 0, contested = s.nonfirst != 0;
-                if (threadIdx.x == 0) s.rows += (unsigned long long)items;
-                __syncthreads();
-                if (had) ++my_rounds;
-                qcur ^= 1;
-                first = false;
-                if (!contested) break;
-            }
-            // step (III a): y(a) -= eps for the columns won in this phase
-            for (int i = threadIdx.x; i < s.nwon; i += blockDim.x) ks[won[i]] += (CB)1;
-            cur ^= 1;
-            __syncthreads();
-        }
-        my_phases += phases;
-        if (failed) {
+        if (c.failed) {
             if (threadIdx.x == 0) record_error(&p.ctl->head, PR_ERR_NO_CONVERGENCE);
             __syncthreads();
             continue;
         }
-
-        // Matching out of the words, completion, duals, cost.
-        int *mb = fl0, *ma = fl1;
-        for (int b = threadIdx.x; b < n; b += blockDim.x) mb[b] = -1;
-        __syncthreads();
-        for (int a = threadIdx.x; a < n; a += blockDim.x) {
-            const unsigned long long w = pw[a];
-            const int b = tag_of(w) > 0 ? row_of(w) : -1;
-            ma[a] = b;
-            if (b >= 0) mb[b] = a;
-        }
-        __syncthreads();
-        // k-th free row (ascending) with the k-th free column (ascending)
-        int *free_b = reinterpret_cast<int *>(ql0);
-        int *free_a = free_b + n;
-        int nfb = 0;
-        for (int base = 0; base < n; base += blockDim.x) {
-            const int b = base + threadIdx.x;
-            const int f = (b < n && mb[b] < 0) ? 1 : 0;
-            const int pos = block_scan_excl(f, s);
-            if (f) free_b[nfb + pos] = b;
-            nfb += s.total;
-            __syncthreads();
-        }
-        int nfa = 0;
-        for (int base = 0; base < n && nfa < nfb; base += blockDim.x) {
-            const int a = base + threadIdx.x;
-            const int f = (a < n && ma[a] < 0) ? 1 : 0;
-            const int pos = block_scan_excl(f, s);
-            if (f && nfa + pos < nfb) free_a[nfa + pos] = a;
-            nfa += s.total;
-            __syncthreads();
-        }
-        for (int k = threadIdx.x; k < nfb; k += blockDim.x) {
-            mb[free_b[k]] = free_a[k];
-            ma[free_a[k]] = free_b[k];
-        }
-        __syncthreads();
-        double acc = 0.0;
-        for (int b = threadIdx.x; b < n; b += blockDim.x) {
-            p.row_to_col[D.v_off + b] = mb[b];
-            p.y_row[D.v_off + b] = yb[b];
-            double c;
-            if (p.points) {
-                c = dist_f64(p.XB + (long long)(D.v_off + b) * p.dim,
-                             p.XA + (long long)(D.v_off + mb[b]) * p.dim, p.dim, p.squared);
-            } else if (p.dt == PR_F64) {
-                c = reinterpret_cast<const double *>(p.C)[D.c_off + (long long)b * n + mb[b]];
-            } else {
-                c = (double)reinterpret_cast<const float *>(p.C)[D.c_off + (long long)b * n + mb[b]];
-            }
-            acc = __dadd_rn(acc, c);
-        }
-        for (int a = threadIdx.x; a < n; a += blockDim.x) {
-            p.col_to_row[D.v_off + a] = ma[a];
-            p.y_col[D.v_off + a] = -(int)ks[a];
-        }
-        // fixed-order tree reduction of the per-thread partial sums
-        double *part = reinterpret_cast<double *>(pw);
-        __syncthreads();
-        part[threadIdx.x] = acc;
-        __syncthreads();
-        for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-            if (threadIdx.x < w) part[threadIdx.x] = __dadd_rn(part[threadIdx.x], part[threadIdx.x + w]);
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) {
-            p.costs[pi] = part[0];
-            p.phases[pi] = phases;
-        }
+        cta_finish<CB>(s, dyn, L, D.n, D.n, part, p.cost_sums, BatchCost{p, D}, p.row_to_col + D.v_off,
+                       p.col_to_row + D.v_off, p.y_row + D.v_off, p.y_col + D.v_off, p.costs + pi);
+        if (threadIdx.x == 0) p.phases[pi] = c.phases;
         __syncthreads();
     }
     if (threadIdx.x == 0) {
         atomicAdd((unsigned long long *)&p.ctl->phases, (unsigned long long)my_phases);
         atomicAdd((unsigned long long *)&p.ctl->rounds, (unsigned long long)my_rounds);
-        atomicAdd(&p.ctl->bytes, s.bytes);
-        atomicAdd(&p.ctl->rows, s.rows);
+        atomicAdd(&p.ctl->bytes, my_bytes);
+        atomicAdd(&p.ctl->rows, my_rows);
     }
-}
-
-size_t bsolve_smem(int n_max, int ldq_max, int threads) {
-    // pw (8) + yb (4) + fl 2x(4) + ql 2x(8) + won (4) per row, keys 2 per column;
-    // rows padded to a multiple of 8 as in k_bsolve; the cost reduction reuses
-    // the front as one double per thread
-    const size_t rows = (size_t)((n_max + 7) & ~7);
-    const size_t state = rows * (8 + 4 + 8 + 16 + 4) + (size_t)ldq_max * 2;
-    const size_t red = (size_t)threads * sizeof(double);
-    return state > red ? state : red;
 }
 
 __global__ void k_binit(BCtl *ctl, unsigned *maxbits, int P) {
@@ -611,7 +364,7 @@ struct Plan {
     std::vector<BDesc> desc;
     std::vector<int> order;
     long long cb_elems = 0, c_elems = 0;
-    int n_max = 0, ldq_max = 0, v_total = 0;
+    int n_max = 0, v_total = 0;
 };
 
 pr_status make_plan(int P, const int32_t *n_host, double eps, Plan &pl) {
@@ -626,7 +379,7 @@ pr_status make_plan(int P, const int32_t *n_host, double eps, Plan &pl) {
         if (n < 1 || n > kMaxN) return fail(PR_ERR_INVALID, "batched: problem %d has n = %d (need 1..%d)", i, n, kMaxN);
         BDesc &d = pl.desc[i];
         d.n = n;
-        d.ldq = (n + 15) & ~15;  // rows start on 16 bytes in either storage type
+        d.ldq = row_stride(n);
         d.cb_off = cb;
         d.c_off = c;
         d.v_off = (int)v;
@@ -636,7 +389,6 @@ pr_status make_plan(int P, const int32_t *n_host, double eps, Plan &pl) {
         c += (long long)n * n;
         v += n;
         pl.n_max = std::max(pl.n_max, n);
-        pl.ldq_max = std::max(pl.ldq_max, d.ldq);
     }
     if (v > (1ll << 30)) return fail(PR_ERR_INVALID, "batched: too many rows in total");
     pl.cb_elems = cb;
@@ -673,9 +425,16 @@ pr_status run_batched(const Source &src, int32_t P, const int32_t *n_host, doubl
     const BLayout L = make_blayout(P, pl.cb_elems);
     if (!ws || ((uintptr_t)ws & 255) || ws_bytes < L.total)
         return fail(PR_ERR_WORKSPACE, "batched: workspace NULL, not 256-byte aligned or < %zu bytes", L.total);
-    int threads = 256, per_sm_want = 0;
+    // Threads per CTA by the largest problem: short rows and few of them want
+    // cheap CTA barriers and many problems per SM, larger problems more warps
+    // (eps = 0.01, ms at 128 / 256 / 512 threads: 512 problems up to 300 rows
+    // 0.95 / 1.40 / 1.44, 300 up to 700: 1.04 / 1.07 / 1.11, 100 up to 1024:
+    // 0.94 / 0.65 / 0.60, 512 up to 2048: 2.69 / 3.04 / 2.67).  The order of
+    // the cost sum stays that of kCostSums partial sums.
+    int threads = pl.n_max <= 400 ? 128 : pl.n_max <= 700 ? 256 : 512, per_sm_want = 0;
+    int cost_sums = kCostSums;
     if (tune) {
-        if (tune->threads) threads = tune->threads;
+        if (tune->threads) cost_sums = threads = tune->threads;
         per_sm_want = tune->ctas_per_sm;
     }
     if (threads != 128 && threads != 256 && threads != 512 && threads != 1024)
@@ -745,8 +504,8 @@ pr_status run_batched(const Source &src, int32_t P, const int32_t *n_host, doubl
     }
     PR_CUDA(cudaGetLastError());
 
-    const size_t smem = bsolve_smem(pl.n_max, pl.ldq_max, threads);
-    if (smem > (size_t)di.max_smem_optin)
+    const size_t smem = CtaLayout(pl.n_max, pl.n_max).total(cb8 ? 1 : 2);
+    if (smem + kCtaStaticSmem > (size_t)di.max_smem_optin)
         return fail(PR_ERR_INVALID, "batched: problem of n = %d does not fit shared memory", pl.n_max);
     // A warp scans a row in 2 KiB steps (a whole row of the largest size
     // for bytes; measured 9.5 % faster than 4 KiB steps on 512 problems of
@@ -764,7 +523,9 @@ pr_status run_batched(const Source &src, int32_t P, const int32_t *n_host, doubl
                                : threads == 256 ? (const void *)k_bsolve<256, 4, uint8_t, false>
                                : threads == 512 ? (const void *)k_bsolve<512, 4, uint8_t, false>
                                                 : (const void *)k_bsolve<1024, 4, uint8_t, false>);
-    PR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // one value for every batch, so that calls from several threads agree
+    PR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)((size_t)di.max_smem_optin - kCtaStaticSmem)));
     int per_sm = 0;
     PR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
     if (per_sm < 1) return fail(PR_ERR_INVALID, "batched: solver CTA does not fit an SM");
@@ -780,7 +541,7 @@ pr_status run_batched(const Source &src, int32_t P, const int32_t *n_host, doubl
     bp.cb = d_cb;
     bp.nprob = P;
     bp.n_max = pl.n_max;
-    bp.ldq_max = pl.ldq_max;
+    bp.cost_sums = cost_sums;
     bp.C = src.C;
     bp.dt = src.dt;
     bp.XA = src.XA;

@@ -10,6 +10,13 @@
 
 namespace prot {
 
+// Row stride of the rounded costs: rows start on 32 bytes in either storage
+// type where the CTA solver may read them (its 32-byte loads), otherwise on 16.
+constexpr int kRowAlign = 32;
+constexpr int kCtaMaxCols = 8000;  // cta_solve.cuh
+constexpr int row_stride(int cols) {
+    return cols <= kCtaMaxCols ? (cols + kRowAlign - 1) & ~(kRowAlign - 1) : (cols + 15) & ~15;
+}
 constexpr uint16_t kPadCost = 0x7FFF;  // cbar of padding columns
 constexpr uint16_t kPadKey = 0x8000;   // k of padding columns: pad sum 0xFFFF never matches
 
@@ -174,6 +181,59 @@ __device__ __forceinline__ unsigned eq_mask8(uint4 c, uint4 k, uint32_t t4) {
          may_match<F7>(c.w, k.w, t4)) == 0u)
         return 0u;
     return eq_mask8_exact(c, k, t4);
+}
+
+// The exact test without a branch, for scans that find a candidate in most
+// vectors: bit j of the result is set iff column j of the vector has cbar + k
+// == target.  Per word 5 operations mark the zero bytes (halves) of z = (c +
+// k) ^ t at their top bit, and one dp4a gathers a word's marks into bits
+// (0x80 per marked byte times a power of two, summed), 27 instructions per
+// 16 bytes against about 70 for the pre-test and eq_mask8_exact together.
+// 16-bit values: cbar + k <= 65534 never carries between halves (padding
+// 0x7FFF + 0x8000).  Bytes with F7: real columns' sums stay below 256 and
+// padding bytes sit above them; otherwise byte_marks masks the carries.
+__device__ __forceinline__ uint32_t half_marks(uint32_t s, uint32_t t2) {
+    const uint32_t z = s ^ t2;
+    return ~(((z & 0x7FFF7FFFu) + 0x7FFF7FFFu) | z) & 0x80008000u;
+}
+template <bool F7>
+__device__ __forceinline__ uint32_t byte_marks_of(uint32_t c, uint32_t k, uint32_t t4) {
+    if (!F7) return byte_marks(c, k, t4);
+    const uint32_t z = (c + k) ^ t4;
+    return ~(((z & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | z) & 0x80808080u;
+}
+template <class CB, bool F7>
+__device__ __forceinline__ unsigned vec_marks(uint4 c, uint4 k, uint32_t t) {
+    if (sizeof(CB) == 1) {
+        uint32_t lo = __dp4a(byte_marks_of<F7>(c.x, k.x, t), 0x08040201u, 0u);
+        lo = __dp4a(byte_marks_of<F7>(c.y, k.y, t), 0x80402010u, lo);
+        uint32_t hi = __dp4a(byte_marks_of<F7>(c.z, k.z, t), 0x08040201u, 0u);
+        hi = __dp4a(byte_marks_of<F7>(c.w, k.w, t), 0x80402010u, hi);
+        return (lo >> 7) | (hi << 1);
+    }
+    uint32_t m = __dp4a(half_marks(c.x + k.x, t), 0x02000100u, 0u);
+    m = __dp4a(half_marks(c.y + k.y, t), 0x08000400u, m);
+    m = __dp4a(half_marks(c.z + k.z, t), 0x20001000u, m);
+    m = __dp4a(half_marks(c.w + k.w, t), 0x80004000u, m);
+    return m >> 7;
+}
+// A test that never misses a candidate: nonzero if some column of the vector
+// may match (16-bit values and F7: exactly if one does).
+__device__ __forceinline__ uint32_t zero_half(uint32_t z) { return (z - 0x00010001u) & ~z & 0x80008000u; }
+template <class CB, bool F7>
+__device__ __forceinline__ uint32_t vec_may_match(uint4 c, uint4 k, uint32_t t) {
+    if (sizeof(CB) == 1)
+        return may_match<F7>(c.x, k.x, t) | may_match<F7>(c.y, k.y, t) | may_match<F7>(c.z, k.z, t) |
+               may_match<F7>(c.w, k.w, t);
+    return zero_half((c.x + k.x) ^ t) | zero_half((c.y + k.y) ^ t) | zero_half((c.z + k.z) ^ t) |
+           zero_half((c.w + k.w) ^ t);
+}
+
+// Read-only 32-byte load (32-byte aligned).
+__device__ __forceinline__ void ld_nc_v8(const void *p, uint4 &a, uint4 &b) {
+    asm volatile("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
+                 : "l"(p));
 }
 
 // Read-only 16-byte load that does not allocate in L1 (streamed rows).
