@@ -47,6 +47,7 @@
 #include "scan_common.cuh"
 #include "quantise.cuh"
 #include "points.cuh"
+#include "cta_solve.cuh"
 
 namespace prot {
 namespace {
@@ -117,7 +118,7 @@ struct Layout {
 Layout make_layout(int nB, int nA, int grid) {
     Layout L;
     Carver c;
-    L.ldq = (nA + 15) & ~15;  // rows start on 16 bytes in either storage type
+    L.ldq = row_stride(nA);
     L.ctl = c.take<Ctl>(1);
     L.cb = c.take<uint16_t>((size_t)nB * L.ldq);  // room for the uint16 form
     L.ka = c.take<uint16_t>(L.ldq);
@@ -153,6 +154,7 @@ struct Params {
     int rule = 0;      // step I: 0 lowest-index columns, 1 seeded start columns (PR_RULE_OFFSET),
                        // 2 Israeli-Itai, 3 the sequential greedy by displacement chains
     void *ii = nullptr;  // PR_RULE_ISRAELI_ITAI's state region
+    int hand = 0;  // k_phases stops at this many free rows, all in the pool, and k_solo goes on (0: never)
 };
 
 // PR_RULE_OFFSET: in phase `phase1` (counted from 1) free row b starts its
@@ -809,7 +811,7 @@ k_phases(Params p, int warps_per_row, int rows_per_group) {
     // With at most two rows per register group (long rows) every free row
     // goes to the pool, which deals them out evenly (measured at n = 10,000:
     // 1-3 % faster than keeping one); shorter rows keep up to a group's worth.
-    const int keep = rows_per_group > 2 ? min(rows_per_group - 1, kKeepMax) : 0;
+    const int keep = rows_per_group > 2 && p.hand == 0 ? min(rows_per_group - 1, kKeepMax) : 0;
     // Every next-phase row goes to the pool and no CTA takes more than kBatch
     // rows in a round (so its donations of a round fit s.don): the barrier
     // places the donations (grid_sync_pool).
@@ -1049,7 +1051,7 @@ k_phases(Params p, int warps_per_row, int rows_per_group) {
         if (threadIdx.x == 0) s.nfl[cur] = 0;
         cur ^= 1;
         pool_size = pool_next_size;
-        if (nf_next <= p.T) {
+        if (nf_next <= p.T || nf_next <= p.hand) {
             if (cta == 0 && threadIdx.x == 0) ctl->free_at_stop = (int)nf_next;
             break;
         }
@@ -1189,6 +1191,85 @@ k_finish(Params p, Src src, int *match_b, int *match_a, int *free_b, int *free_a
         __syncthreads();
     }
     if (threadIdx.x == 0) *cost = part[0];
+}
+
+// ---------------------------------------------------------------------------
+// k_solo: phases, completion and cost of one problem on one CTA
+// (cta_solve.cuh).
+// ---------------------------------------------------------------------------
+constexpr int kSoloThreads = 512;
+
+__global__ void k_solo_init(Ctl *c) {
+    memset(c, 0, sizeof(Ctl));
+    c->head.magic = kWsMagic;
+}
+
+// RESUME: the first phases ran in k_phases, which stopped at hand_rows free
+// rows: the state is taken over from its words, keys, duals and row pool.
+template <class CB, bool F7, bool RESUME, class Src>
+__global__ void __launch_bounds__(kSoloThreads)
+k_solo(Params p, Src src, int *match_b, int *match_a, int *y_col, double *cost) {
+    extern __shared__ __align__(16) unsigned char dyn[];
+    __shared__ CtaShared s;
+    __shared__ double part[kFinThreads];
+    Ctl *ctl = p.ctl;
+    if (ld_relaxed_s32(&ctl->head.err) != 0) return;  // a cost outside [0, 1], or the first phases stopped
+    const CtaLayout L(p.nB, p.nA);
+    const CtaState<CB> st(dyn, L);
+    CtaCounts c = {0, 0, 0, 0, false};
+    int nf = p.nB;
+    if (RESUME) {
+        c.phases = ctl->phases;
+        c.rounds = ctl->rounds;
+        c.barriers = (long long)ctl->barriers;
+        nf = ctl->free_at_stop;
+        for (int a = threadIdx.x; a < p.ldq; a += blockDim.x) {
+            const unsigned k = p.ka[a];
+            st.ks[a] = sizeof(CB) == 1 && k > 0xFFu ? (CB)0xFF : (CB)k;
+            if (a < p.nA) {
+                const unsigned long long w = p.prop[a];
+                st.pw[a] = tag_of(w) > 0 ? 0x10000u | (0xFFFFu - (unsigned)row_of(w)) : 0u;
+            }
+        }
+        for (int b = threadIdx.x; b < p.nB; b += blockDim.x) st.y[b] = (uint16_t)p.y_b[b];
+        const int2 *pool = p.pool + (size_t)(c.phases & 1) * p.nB;
+        if (nf > p.T)
+            for (int i = threadIdx.x; i < nf; i += blockDim.x) {
+                const int2 e = pool[i];
+                st.la[i] = e.x | ((e.y < 0 ? -1 - e.y : 0) << kCtaRowBits);
+            }
+    } else {
+        cta_init(s, st, p.nB, p.nA, p.ldq);
+    }
+    cta_phases<4, CB, F7, true>(s, st, static_cast<const CB *>(p.cb), p.nB, p.nA, p.ldq, p.T, p.phase_cap,
+                                RESUME ? 1u : 0u, nf, c);
+    if (threadIdx.x == 0) {
+        ctl->phases = c.phases;
+        ctl->rounds = c.rounds;
+        ctl->barriers = (unsigned long long)c.barriers;
+        ctl->free_at_stop = c.free_at_stop;
+        ctl->bytes += s.bytes;
+        ctl->rows += s.rows;
+        ctl->cells += s.cells;
+        if (c.failed) record_error(&ctl->head, PR_ERR_NO_CONVERGENCE);
+    }
+    if (c.failed) return;
+    cta_finish<CB>(s, dyn, L, p.nB, p.nA, part, kFinThreads, src, match_b, match_a, p.y_b, y_col, cost);
+}
+
+template <bool RESUME, class Src>
+pr_status launch_solo(const Params &p, const Src &src, bool cb8, bool f7, int *match_b, int *match_a, int *y_col,
+                      double *cost, cudaStream_t st) {
+    const size_t smem = CtaLayout(p.nB, p.nA).total(cb8 ? 1 : 2);
+    const auto fn = !cb8 ? k_solo<uint16_t, false, RESUME, Src>
+                    : f7 ? k_solo<uint8_t, true, RESUME, Src>
+                         : k_solo<uint8_t, false, RESUME, Src>;
+    // one value for every size, so that calls from several threads agree
+    const int smem_max = (int)((size_t)device_info().max_smem_optin - kCtaStaticSmem);
+    PR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
+    fn<<<1, kSoloThreads, smem, st>>>(p, src, match_b, match_a, y_col, cost);
+    PR_CUDA(cudaGetLastError());
+    return PR_OK;
 }
 
 // ---------------------------------------------------------------------------
@@ -1412,29 +1493,64 @@ pr_status phase_cfg(PhaseCfg &cfg) {
 }
 
 // The phase loop runs in one thread-block cluster (barriers through
-// distributed shared memory, about a third of a grid barrier's latency) or
-// on the whole grid (one CTA per SM, barriers through L2).  PR_PHASE_MODE =
-// "grid" or "cluster" forces one; otherwise the cluster runs problems of up
-// to kClusterMaxRows rows with floor(1/eps) > kClusterMinK.
+// distributed shared memory, about a third of a grid barrier's latency), on
+// the whole grid (one CTA per SM, barriers through L2), on one CTA, or on the
+// grid and then on one CTA.  PR_PHASE_MODE = "grid", "cluster", "solo" or
+// "hand" forces one (the last two where they fit).
 // Cluster mode also needs at least kMinSlots row slots next to the keys.
 constexpr int kMinSlots = 4;
 
-// Measured on GB300 (eps = 0.01): the cluster is ahead up to a few thousand
-// rows (n = 2000: 15 %, n = 4000: 6 %); at n = 10,000 the 16 SMs' scan
-// throughput falls behind the whole grid's (37 % slower).
+// The cluster runs by itself only for the offset rule, up to a few thousand
+// rows at floor(1/eps) > 20 (its two jobs per row keep 16 SMs busy; at larger
+// eps a solve is one phase of many rounds with many rows, where the whole
+// grid's scans win).  The lowest-index rule takes one CTA for its small rounds
+// instead (use_cta), and where it does not the grid is ahead (ms, cluster /
+// grid: n = 3000, eps = 0.02 0.714 / 0.655; n = 4000, eps = 0.02 0.832 /
+// 0.730, eps = 0.01 2.94 / 2.79).
 constexpr int kClusterMaxRows = 4096;
-// ... and only when floor(1/eps) > 20: at larger eps a solve is one phase of
-// many rounds with many rows, where the whole grid's scans win (eps = 0.1:
-// n = 1000 0.152 vs 0.169 ms, n = 3000 0.333 vs 0.505 ms, grid vs cluster;
-// eps = 0.01: 8.24 vs 7.42 ms and 1.97 vs 1.99 ms).
 constexpr long long kClusterMinK = 20;
 
-bool use_cluster(const PhaseCfg &cfg, int nslots, int n_rows, long long K) {
+bool use_cluster(const PhaseCfg &cfg, int nslots, int n_rows, long long K, int rule) {
     if (cfg.cluster < 1 || nslots < kMinSlots) return false;
     const char *m = getenv("PR_PHASE_MODE");
     if (m && strcmp(m, "grid") == 0) return false;
     if (m && strcmp(m, "cluster") == 0) return true;
-    return n_rows <= kClusterMaxRows && K > kClusterMinK;
+    return rule == PR_RULE_OFFSET && n_rows <= kClusterMaxRows && K > kClusterMinK;
+}
+
+// Small problems.  A round of the grid costs about 4.3 us whatever it does (a
+// grid barrier and four or five dependent L2 trips); on one CTA with its
+// state in shared memory it costs 0.9 us with a few rows, and grows with the
+// rows, since one SM scans them all.  So one CTA runs problems of up to
+// kSoloMaxRows rows from the start, and for larger ones the grid runs the
+// first, crowded phases and one CTA the rest, from the first phase with at
+// most kHandRows free rows (fewer with long rows: kHandBytes of rounded costs
+// in all).  Where T is not below that, the grid runs alone.  Solve time, ms,
+// eps = 0.01 / 0.003, one CTA / take-over / grid: n = 300: 0.46 / 0.47 / 1.44,
+// 12.6 / 12.9 / 54; n = 1000: 1.61 / 1.60 / 3.93, 8.8 / 8.6 / 24.7; n = 2000:
+// 1.70 / 1.44 / 2.23, 16.4 / 14.3 / 30.6; n = 4000: 3.85 / 2.53 / 2.79, 36 /
+// 24.0 / 27.4; 1000 x 1500: 0.23 / 0.13 / 0.17, 0.72 / 0.41 / 0.63.  Half or
+// twice the rows or bytes was slower; rows past kHandRowBytes as well (n =
+// 6000 in 16 bits: 43.0 against 41.8).
+constexpr int kSoloMaxRows = 384;
+constexpr int kHandRows = 64, kHandBytes = 256 * 1024, kHandRowBytes = 8192;
+
+// Whether one CTA runs the problem from the start (solo), or takes over from
+// the grid once at most `hand` rows are free (0: never).
+void use_cta(const Params &p, size_t smem_max, int key_bytes, bool &solo, int &hand) {
+    solo = false;
+    hand = 0;
+    if (p.rule != PR_RULE_LOWEST || p.profile || p.nA > kCtaMaxCols) return;
+    if (CtaLayout(p.nB, p.nA).total(key_bytes) + kCtaStaticSmem > smem_max) return;
+    const char *m = getenv("PR_PHASE_MODE");
+    if (m && (strcmp(m, "grid") == 0 || strcmp(m, "cluster") == 0)) return;
+    if (m ? strcmp(m, "solo") == 0 : p.nB <= kSoloMaxRows) {
+        solo = true;
+        return;
+    }
+    const int row_bytes = p.ldq * key_bytes;
+    const int rows = std::min(kHandRows, kHandBytes / row_bytes);
+    if (row_bytes <= kHandRowBytes && rows > p.T) hand = rows;
 }
 
 // Row scans of the grid form: a CTA with more jobs than one register group
@@ -1564,7 +1680,10 @@ pr_status launch_solve(Params &p, const CostSource &src, double eps, const Phase
     const bool f7 = cb8 && K <= kMaxCbar7;  // and cbar + key < 256 on every real column
 
     const DeviceInfo &di = device_info();
-    k_init<<<di.sms * 2, 256, 0, st>>>(p, row_to_col);
+    bool solo;
+    use_cta(p, cfg.smem, cb8 ? 1 : 2, solo, p.hand);
+    if (solo) k_solo_init<<<1, 1, 0, st>>>(p.ctl);
+    else k_init<<<di.sms * 2, 256, 0, st>>>(p, row_to_col);
     PR_CUDA(cudaGetLastError());
     const long long groups = (long long)n_rows * (p.ldq >> 3);
     const long long want = groups / 256 + 1;
@@ -1607,8 +1726,10 @@ pr_status launch_solve(Params &p, const CostSource &src, double eps, const Phase
     const int kb = cb8 ? 1 : 2;  // bytes per key in the shared-memory copy
     const size_t slot_room = cfg.smem > slots_offset(p.ldq, kb) ? cfg.smem - slots_offset(p.ldq, kb) : 0;
     p.nslots = (int)std::min<size_t>((size_t)kWarps, slot_room / (size_t)p.slot_bytes);
-    const bool cluster = p.rule <= PR_RULE_OFFSET && use_cluster(cfg, p.nslots, n_rows, K);
-    if (p.rule == PR_RULE_SEQUENTIAL) {
+    const bool cluster = !solo && p.hand == 0 && p.rule <= PR_RULE_OFFSET && use_cluster(cfg, p.nslots, n_rows, K, p.rule);
+    if (solo) {
+        // below
+    } else if (p.rule == PR_RULE_SEQUENTIAL) {
         // the phase's keys live in shared memory, one per column (the size
         // was checked by pr_assign_rule)
         const size_t ksm = (size_t)p.ldq * (cb8 ? 1 : 2);
@@ -1662,14 +1783,26 @@ pr_status launch_solve(Params &p, const CostSource &src, double eps, const Phase
         const size_t smem = sl ? slots_offset(p.ldq, kb) + (size_t)p.nslots * p.slot_bytes : smem_bytes(p.ldq, kb);
         PR_CUDA(cudaLaunchCooperativeKernel(fn, dim3(cfg.grid), dim3(kThreads), args, smem, st));
     }
+    if (solo || p.hand) {
+        const auto run = [&](auto cost_src) {
+            return solo ? launch_solo<false>(p, cost_src, cb8, f7, row_to_col, col_to_row, y_col, cost, st)
+                        : launch_solo<true>(p, cost_src, cb8, f7, row_to_col, col_to_row, y_col, cost, st);
+        };
+        const pr_status rc = src.points     ? run(PointsCost{src.XA, src.XB, src.dim, src.squared})
+                             : dt == PR_F64 ? run(MatrixCost<double>{(const double *)C, ldc})
+                                            : run(MatrixCost<float>{(const float *)C, ldc});
+        if (rc != PR_OK) return rc;
+    }
     if (ev0 && ev1) PR_CUDA(cudaEventRecord(ev1, st));
 
-    k_decode<<<di.sms * 2, 256, 0, st>>>(p, row_to_col, col_to_row, y_col);
+    if (!solo && !p.hand) k_decode<<<di.sms * 2, 256, 0, st>>>(p, row_to_col, col_to_row, y_col);
     PR_CUDA(cudaGetLastError());
     // completion scratch: the first CTA's list region (free after the loop)
     int *free_b = p.lists;
     int *free_a = p.lists + n_rows;
-    if (src.points)
+    if (solo || p.hand) {
+        // done by k_solo
+    } else if (src.points)
         k_finish<PointsCost><<<1, kFinThreads, 0, st>>>(p, PointsCost{src.XA, src.XB, src.dim, src.squared},
                                                          row_to_col, col_to_row, free_b, free_a, cost);
     else if (dt == PR_F64)
@@ -1691,7 +1824,7 @@ pr_status launch_solve(Params &p, const CostSource &src, double eps, const Phase
         stats->cells_examined = (int64_t)h.cells;
         stats->free_at_stop = h.free_at_stop;
         stats->threshold = p.T;
-        stats->loop_ctas = cluster ? cfg.cluster : cfg.grid;
+        stats->loop_ctas = solo ? 1 : cluster ? cfg.cluster : cfg.grid;
         stats->loop_cluster = cluster ? 1 : 0;
         stats->barriers = (int64_t)h.barriers;
         if (h.head.err != 0)
@@ -1914,7 +2047,7 @@ struct NoAllocLayout {
 NoAllocLayout make_noalloc_layout(int nB, int nA) {
     NoAllocLayout L;
     Carver c;
-    L.ldq = (nA + 15) & ~15;  // rows start on 16 bytes in either storage type
+    L.ldq = row_stride(nA);
     L.ctl = c.take<Ctl>(1);
     L.cb = c.take<uint16_t>((size_t)nB * L.ldq);  // room for the uint16 form
     L.ka = c.take<uint16_t>(L.ldq);
