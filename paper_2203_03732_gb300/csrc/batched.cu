@@ -112,22 +112,10 @@ __device__ __forceinline__ int problem_of_row(const BDesc *d, int P, int r) {
     return lo;
 }
 
-// Columns per lane in flight per step of the matrix rounding: 2 KiB per warp
-// (16 FP32 or 8 FP64 values a lane), 64 KiB per SM at 32 warps, enough to
-// cover the load latency at the copy rate (1 KiB per warp reached 3.4 TB/s).
-template <class T> constexpr int kRowUnroll = sizeof(T) == 8 ? 8 : 16;
-// Columns per lane in flight per step of the points kernels.
-constexpr int kPtUnroll = 4;
-
-__device__ __forceinline__ uint32_t quantise_val(double x, const EpsSplit &e) {
-    const unsigned long long bits = __double_as_longlong(x);
-    return quantise_bits((uint32_t)(bits >> 32), (uint32_t)bits, e);
-}
-__device__ __forceinline__ uint32_t quantise_val(float x, const EpsSplit &e) {
-    return quantise_fbits(__float_as_uint(x), e);
-}
-
-// Eq. (1) on the packed matrices, exactly as k_quantise does for one problem.
+// Eq. (1) on the packed matrices, a warp per row (round_chunk): about 8
+// instructions per cost and 64 bytes in flight per lane.  512 problems (3.17
+// GB of FP32 read, 0.80 GB written): 1.06 ms -> 0.71 ms; it was bound by the 25
+// instructions a cost took one at a time.
 template <class T, class CB>
 __global__ void __launch_bounds__(256, 4) k_bquant_matrix(const T *__restrict__ C, const BDesc *__restrict__ d, int P, int total_rows,
                                 EpsSplit e, CB *__restrict__ cb, WsHead *head) {
@@ -135,149 +123,153 @@ __global__ void __launch_bounds__(256, 4) k_bquant_matrix(const T *__restrict__ 
     const int nw = (gridDim.x * blockDim.x) >> 5;
     bool bad = false;
     for (int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < total_rows; r += nw) {
-        const int i = problem_of_row(d, P, r);
-        const BDesc D = d[i];
+        const BDesc D = d[problem_of_row(d, P, r)];
         const int b = r - D.v_off;
         const T *row = C + D.c_off + (long long)b * D.n;
         CB *out = cb + D.cb_off + (long long)b * D.ldq;
-        for (int a0 = 0; a0 < D.ldq; a0 += 32 * kRowUnroll<T>) {
-            T x[kRowUnroll<T>];
-#pragma unroll
-            for (int u = 0; u < kRowUnroll<T>; ++u) {
-                const int a = a0 + 32 * u + lane;
-                x[u] = a < D.n ? __ldg(row + a) : (T)0;
-            }
-#pragma unroll
-            for (int u = 0; u < kRowUnroll<T>; ++u) {
-                const int a = a0 + 32 * u + lane;
-                if (a >= D.ldq) break;
-                uint32_t q = kPadOf<CB>;
-                if (a < D.n) {
-                    q = quantise_val(x[u], e);
-                    if (q == 0xFFFFFFFFu) {
-                        bad = true;
-                        q = 0;
-                    }
-                }
-                out[a] = (CB)q;
-            }
-        }
+        for (int c0 = 0; c0 < D.ldq; c0 += kRoundCols<T>) round_chunk<T, CB>(row, D.n, D.ldq, c0, e, out, lane, bad);
     }
     if (bad) record_error(head, PR_ERR_INVALID);
 }
 
 // ---------------------------------------------------------------------------
-// Costs from points (points.cuh): c = RN32(d / max d) per problem.
+// Costs from points (points.cuh): c = RN32(d / max d) per problem.  A warp
+// takes kPtRows global rows (cut at problem boundaries) and, step by step, 4
+// consecutive columns a lane, so a column's coordinates are loaded once per
+// kPtRows pairs and the rounded costs are stored 4 (16-bit storage: 8) bytes at
+// a time; the squared sum keeps the operation order of dist_f32.  DIM = 0: any
+// dimension, one pair at a time.  64 clouds of 4096 3-D points (1.07 G pairs):
+// largest distance 0.96 -> 0.35 ms, rounding 2.20 -> 0.82 ms (three loads and about
+// 60 instructions a pair before).
 // ---------------------------------------------------------------------------
-// d(b, a) from b's coordinates held in registers, in the operation order of
-// dist_f32 (ascending k, one IEEE operation at a time); DIM > 0 is the
-// dimension known at compile time.
-template <int DIM>
-__device__ __forceinline__ float dist_regs(const float (&xb)[DIM], const float (&xa)[DIM], int squared) {
-    float acc = 0.0f;
-#pragma unroll
-    for (int k = 0; k < DIM; ++k) {
-        const float t = __fsub_rn(xb[k], xa[k]);
-        const float sq = __fmul_rn(t, t);
-        acc = k == 0 ? sq : __fadd_rn(acc, sq);
+constexpr int kPtRows = 8;
+
+// Calls body(problem, first global row, rows) for each run of rows that this
+// warp takes.
+template <class Body>
+__device__ __forceinline__ void point_tiles(const BDesc *__restrict__ d, int P, int total_rows, const Body &body) {
+    const int nw = (gridDim.x * blockDim.x) >> 5;
+    for (int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; (long long)t * kPtRows < total_rows; t += nw) {
+        const int end = min(total_rows, (t + 1) * kPtRows);
+        for (int r = t * kPtRows; r < end;) {
+            const int i = problem_of_row(d, P, r);
+            const int stop = min(end, d[i].v_off + d[i].n);
+            body(i, r, stop - r);
+            r = stop;
+        }
     }
-    return squared ? acc : __fsqrt_rn(acc);
 }
 
-// Largest distance of every problem: a warp's maximum over one row, then one
-// atomic per row (non-negative floats order like their bit patterns).  DIM =
-// 0: any dimension, one column at a time; DIM > 0: each lane loads the
-// coordinates of kPtUnroll columns before it computes.
+// The squared sums of one row point against a lane's 4 column points.
 template <int DIM>
-__global__ void k_bpoints_max(const float *__restrict__ XA, const float *__restrict__ XB, int dim,
-                              int squared, const BDesc *__restrict__ d, int P, int total_rows,
-                              unsigned *maxbits) {
+__device__ __forceinline__ void sq_group4(const float (&xb)[DIM], const float (&xa)[4][DIM], float (&sq)[4]) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        float acc = 0.0f;
+#pragma unroll
+        for (int k = 0; k < DIM; ++k) {
+            const float t = __fsub_rn(xb[k], xa[j][k]);
+            const float q = __fmul_rn(t, t);
+            acc = k == 0 ? q : __fadd_rn(acc, q);
+        }
+        sq[j] = acc;
+    }
+}
+
+template <int DIM>
+__device__ __forceinline__ void load_points(const float *__restrict__ XB, int r, int rows, float (&xb)[kPtRows][DIM]) {
+#pragma unroll
+    for (int q = 0; q < kPtRows; ++q)
+#pragma unroll
+        for (int k = 0; k < DIM; ++k) xb[q][k] = __ldg(XB + (long long)(r + min(q, rows - 1)) * DIM + k);
+}
+template <int DIM>
+__device__ __forceinline__ void load_columns(const float *__restrict__ XA, const BDesc &D, int a, float (&xa)[4][DIM]) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j)  // columns past the last repeat it
+#pragma unroll
+        for (int k = 0; k < DIM; ++k) xa[j][k] = __ldg(XA + (long long)(D.v_off + min(a + j, D.n - 1)) * DIM + k);
+}
+
+// Largest squared sum of every problem (the IEEE root is non-decreasing, so
+// the root of the largest sum is the largest root): one atomic per run of
+// rows (non-negative floats order like their bit patterns).
+template <int DIM>
+__global__ void __launch_bounds__(256, 4) k_bpoints_max(const float *__restrict__ XA, const float *__restrict__ XB, int dim,
+                              const BDesc *__restrict__ d, int P, int total_rows, unsigned *maxbits) {
     const int lane = threadIdx.x & 31;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    for (int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < total_rows; r += nw) {
-        const int i = problem_of_row(d, P, r);
+    point_tiles(d, P, total_rows, [&](int i, int r, int rows) {
         const BDesc D = d[i];
-        const float *xbp = XB + (long long)r * dim;  // row b of problem i is global row r
         float m = 0.0f;
-        if (DIM == 0) {
-            for (int a = lane; a < D.n; a += 32)
-                m = fmaxf(m, dist_f32(xbp, XA + (long long)(D.v_off + a) * dim, dim, squared));
+        if constexpr (DIM == 0) {
+            for (int q = 0; q < rows; ++q)
+                for (int a = lane; a < D.n; a += 32)
+                    m = fmaxf(m, dist_f32(XB + (long long)(r + q) * dim, XA + (long long)(D.v_off + a) * dim, dim, 1));
         } else {
-            constexpr int DD = DIM > 0 ? DIM : 1;
-            float xb[DD];
+            float xb[kPtRows][DIM];
+            load_points<DIM>(XB, r, rows, xb);  // rows past the run's last repeat it
+            for (int a = 4 * lane; a < D.n; a += 128) {
+                float xa[4][DIM];
+                load_columns<DIM>(XA, D, a, xa);
 #pragma unroll
-            for (int k = 0; k < DD; ++k) xb[k] = xbp[k];
-            for (int a0 = 0; a0 < D.n; a0 += 32 * kPtUnroll) {
-                float xa[kPtUnroll][DD];
-#pragma unroll
-                for (int u = 0; u < kPtUnroll; ++u) {
-                    const int a = a0 + 32 * u + lane;
-                    const float *q = XA + (long long)(D.v_off + (a < D.n ? a : 0)) * DD;
-#pragma unroll
-                    for (int k = 0; k < DD; ++k) xa[u][k] = __ldg(q + k);
+                for (int q = 0; q < kPtRows; ++q) {
+                    float sq[4];
+                    sq_group4<DIM>(xb[q], xa, sq);
+                    m = fmaxf(m, fmaxf(fmaxf(sq[0], sq[1]), fmaxf(sq[2], sq[3])));
                 }
-#pragma unroll
-                for (int u = 0; u < kPtUnroll; ++u)
-                    if (a0 + 32 * u + lane < D.n) m = fmaxf(m, dist_regs<DD>(xb, xa[u], squared));
             }
         }
         const unsigned mx = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(m));
         if (lane == 0) atomicMax(maxbits + i, mx);
-    }
+    });
 }
 
 template <int DIM, class CB>
-__global__ void k_bpoints_quant(const float *__restrict__ XA, const float *__restrict__ XB, int dim,
+__global__ void __launch_bounds__(256, 3) k_bpoints_quant(const float *__restrict__ XA, const float *__restrict__ XB, int dim,
                                 int squared, const BDesc *__restrict__ d, int P, int total_rows,
                                 const unsigned *__restrict__ maxbits, EpsSplit e, CB *__restrict__ cb) {
     const int lane = threadIdx.x & 31;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    for (int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < total_rows; r += nw) {
-        const int i = problem_of_row(d, P, r);
+    point_tiles(d, P, total_rows, [&](int i, int r, int rows) {
         const BDesc D = d[i];
-        const int b = r - D.v_off;
-        const float M = __uint_as_float(maxbits[i]);
-        const float *xbp = XB + (long long)r * dim;
-        CB *out = cb + D.cb_off + (long long)b * D.ldq;
-        if (DIM == 0) {
-            for (int a = lane; a < D.ldq; a += 32) {
-                uint32_t q = kPadOf<CB>;
-                if (a < D.n) {
-                    const float dd = dist_f32(xbp, XA + (long long)(D.v_off + a) * dim, dim, squared);
-                    const float c = M > 0.0f ? __fdiv_rn(dd, M) : 0.0f;
-                    q = quantise_fbits(__float_as_uint(c), e);
-                }
-                out[a] = (CB)q;
-            }
-        } else {
-            constexpr int DD = DIM > 0 ? DIM : 1;
-            float xb[DD];
-#pragma unroll
-            for (int k = 0; k < DD; ++k) xb[k] = xbp[k];
-            for (int a0 = 0; a0 < D.ldq; a0 += 32 * kPtUnroll) {
-                float xa[kPtUnroll][DD];
-#pragma unroll
-                for (int u = 0; u < kPtUnroll; ++u) {
-                    const int a = a0 + 32 * u + lane;
-                    const float *q = XA + (long long)(D.v_off + (a < D.n ? a : 0)) * DD;
-#pragma unroll
-                    for (int k = 0; k < DD; ++k) xa[u][k] = __ldg(q + k);
-                }
-#pragma unroll
-                for (int u = 0; u < kPtUnroll; ++u) {
-                    const int a = a0 + 32 * u + lane;
-                    if (a >= D.ldq) break;
-                    uint32_t q = kPadOf<CB>;
+        const PointsScale ps = points_scale(maxbits[i], squared, e);
+        CB *out = cb + D.cb_off + (long long)(r - D.v_off) * D.ldq;
+        if constexpr (DIM == 0) {
+            for (int q = 0; q < rows; ++q)
+                for (int a = lane; a < D.ldq; a += 32) {
+                    uint32_t h = kPadOf<CB>;
                     if (a < D.n) {
-                        const float dd = dist_regs<DD>(xb, xa[u], squared);
-                        const float c = M > 0.0f ? __fdiv_rn(dd, M) : 0.0f;
-                        q = quantise_fbits(__float_as_uint(c), e);
+                        const float dd =
+                            dist_f32(XB + (long long)(r + q) * dim, XA + (long long)(D.v_off + a) * dim, dim, squared);
+                        const float c = ps.M > 0.0f ? __fdiv_rn(dd, ps.M) : 0.0f;
+                        h = quantise_fbits(__float_as_uint(c), e);
                     }
-                    out[a] = (CB)q;
+                    out[(long long)q * D.ldq + a] = (CB)h;
+                }
+        } else {
+            float xb[kPtRows][DIM];
+            load_points<DIM>(XB, r, rows, xb);
+            for (int a = 4 * lane; a < D.ldq; a += 128) {
+                float xa[4][DIM];
+                load_columns<DIM>(XA, D, a, xa);
+#pragma unroll
+                for (int q = 0; q < kPtRows; ++q) {
+                    if (q >= rows) break;
+                    float sq[4];
+                    uint32_t h[4];
+                    sq_group4<DIM>(xb[q], xa, sq);
+                    quantise_points<4>(sq, squared, ps, e, h, [](float, uint32_t k) { return k; });
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if (a + j >= D.n) h[j] = kPadOf<CB>;
+                    CB *o = out + (long long)q * D.ldq + a;
+                    if (sizeof(CB) == 1)
+                        *reinterpret_cast<uint32_t *>(o) = pack_bytes(h[0], h[1], h[2], h[3]);
+                    else
+                        *reinterpret_cast<uint2 *>(o) = make_uint2(pack_halves(h[0], h[1]), pack_halves(h[2], h[3]));
                 }
             }
         }
-    }
+    });
 }
 
 // ---------------------------------------------------------------------------
@@ -464,8 +456,7 @@ pr_status run_batched(const Source &src, int32_t P, const int32_t *n_host, doubl
     const int qgrid = std::max(1, std::min(di.sms * 4, (pl.v_total + 7) / 8));
     if (src.points) {
         // two and three dimensions have their own kernels (coordinates in
-        // registers, several columns' loads in flight); any other runs the
-        // column-at-a-time form
+        // registers); any other runs one pair at a time
         const int D = src.dim == 2 ? 2 : src.dim == 3 ? 3 : 0;
         const void *kmax = D == 2 ? (const void *)k_bpoints_max<2> : D == 3 ? (const void *)k_bpoints_max<3>
                                                                               : (const void *)k_bpoints_max<0>;
@@ -479,14 +470,16 @@ pr_status run_batched(const Source &src, int32_t P, const int32_t *n_host, doubl
         const float *xa_ = src.XA, *xb_ = src.XB;
         const BDesc *dd_ = d_desc;
         unsigned *mx_ = d_max;
-        void *amax[] = {(void *)&xa_, (void *)&xb_, (void *)&dim_, (void *)&sq_, (void *)&dd_, (void *)&P_,
-                        (void *)&rows_, (void *)&mx_};
-        PR_CUDA(cudaLaunchKernel(kmax, dim3(qgrid), dim3(256), amax, 0, st));
+        // a warp per kPtRows rows
+        const int pgrid = std::max(1, std::min(di.sms * 4, (pl.v_total + 8 * kPtRows - 1) / (8 * kPtRows)));
+        void *amax[] = {(void *)&xa_, (void *)&xb_, (void *)&dim_, (void *)&dd_, (void *)&P_, (void *)&rows_,
+                        (void *)&mx_};
+        PR_CUDA(cudaLaunchKernel(kmax, dim3(pgrid), dim3(256), amax, 0, st));
         const unsigned *cmx_ = d_max;
         void *cbp_ = d_cb;
         void *aq[] = {(void *)&xa_, (void *)&xb_, (void *)&dim_, (void *)&sq_, (void *)&dd_, (void *)&P_,
                       (void *)&rows_, (void *)&cmx_, (void *)&e, (void *)&cbp_};
-        PR_CUDA(cudaLaunchKernel(kq, dim3(qgrid), dim3(256), aq, 0, st));
+        PR_CUDA(cudaLaunchKernel(kq, dim3(pgrid), dim3(256), aq, 0, st));
     } else if (src.dt == PR_F64) {
         if (cb8)
             k_bquant_matrix<double, uint8_t><<<qgrid, 256, 0, st>>>((const double *)src.C, d_desc, P, pl.v_total, e,

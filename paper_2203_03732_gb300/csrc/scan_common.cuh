@@ -121,6 +121,115 @@ __device__ __forceinline__ uint32_t quantise_fbits(uint32_t fb, const EpsSplit &
     return k;
 }
 
+// ---------------------------------------------------------------------------
+// Eq. (1) for a group of N values: 7 (FP32) to 9 (FP64) instructions each on
+// the way that nearly all take, against about 25 for quantise_bits one value
+// at a time, which bound the rounding kernels by instructions, not memory.
+//
+// t = 2^23 + v * scale rounded down has floor(v * scale) in its low bits (the
+// sum's unit is 1, and the product is not rounded first); d = v * scale -
+// floor - 1/2 tells how near an integer the estimate is.  A value whose |d|
+// is within `near` of 1/2, or whose bits lie outside the range that the
+// estimate covers, is settled by `exact(j)`; one test covers the group.
+// Only the low 8 or 16 bits of h[j] are the result.
+// ---------------------------------------------------------------------------
+template <int N, class Exact>
+__device__ __forceinline__ void floor_group(const float (&v)[N], float scale, float near, bool out_of_range,
+                                            uint32_t (&h)[N], const Exact &exact) {
+    float d[N], far = 0.0f;
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        const float t = __fmaf_rd(v[j], scale, 8388608.0f);
+        d[j] = __fmaf_rn(v[j], scale, __fsub_rn(8388607.5f, t));  // 2^23 - 1/2 - t is exact
+        far = fmaxf(far, fabsf(d[j]));
+        h[j] = __float_as_uint(t);
+    }
+    if (out_of_range || !(far <= 0.5f - near)) {
+#pragma unroll
+        for (int j = 0; j < N; ++j)
+            if (out_of_range || !(fabsf(d[j]) <= 0.5f - near)) h[j] = exact(j);
+    }
+}
+
+// FP32 costs.  The estimate's error is below (floor(1/eps) + 1) * 2^-23 (the
+// rounding of 1/eps), inside e.win.
+template <int N>
+__device__ __forceinline__ void quantise_group(const float (&c)[N], const EpsSplit &e, uint32_t (&h)[N], bool &bad) {
+    uint32_t top = 0;
+#pragma unroll
+    for (int j = 0; j < N; ++j) top = max(top, __float_as_uint(c[j]));
+    floor_group<N>(c, e.inv, e.win, top > 0x3F800000u, h, [&](int j) {
+        const uint32_t q = quantise_fbits(__float_as_uint(c[j]), e);
+        if (q == 0xFFFFFFFFu) bad = true;
+        return q == 0xFFFFFFFFu ? 0u : q;
+    });
+}
+
+// FP64 costs: for 2^-127 <= c < 1 the exponent's low 7 bits and the mantissa's
+// leading 23 are those of c truncated to FP32 (relative error below 2^-23), so
+// with the rounding of 1/eps the error is below (floor(1/eps) + 1) * 1.5 *
+// 2^-23, inside e.win.  Everything else, 0 and 1 among it, is out of range.
+template <int N>
+__device__ __forceinline__ void quantise_group(const double (&c)[N], const EpsSplit &e, uint32_t (&h)[N], bool &bad) {
+    float f[N];
+    uint32_t top = 0;
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        const unsigned long long b = (unsigned long long)__double_as_longlong(c[j]);
+        const uint32_t hi = (uint32_t)(b >> 32), lo = (uint32_t)b;
+        f[j] = __uint_as_float(__funnelshift_l(lo, hi, 3) & 0x3FFFFFFFu);
+        top = max(top, hi - 0x38000000u);
+    }
+    floor_group<N>(f, e.inv, e.win, top >= 0x07F00000u, h, [&](int j) {
+        const unsigned long long b = (unsigned long long)__double_as_longlong(c[j]);
+        const uint32_t q = quantise_bits((uint32_t)(b >> 32), (uint32_t)b, e);
+        if (q == 0xFFFFFFFFu) bad = true;
+        return q == 0xFFFFFFFFu ? 0u : q;
+    });
+}
+
+// Costs from points: c = RN32(dist / M), dist the squared sum sq or its IEEE
+// root, M the largest.  scale = RN32(e.inv / M).  Against the exact c / eps
+// the estimate is off by at most 6 * 2^-24 of it (the two roundings of c, the
+// approximate root's 2^-23, the two of the scale), 0.75 e.win; the test takes
+// twice e.win.  Out of range: an M whose scale could overflow or lose bits
+// (all values then, M is the same for all), and NaN.  exact_cost(dist, q) is
+// called with the exact way's distance and result and returns what to store.
+struct PointsScale {
+    float M, scale;
+    bool wide;
+};
+__device__ __forceinline__ PointsScale points_scale(uint32_t max_sq_bits, int squared, const EpsSplit &e) {
+    PointsScale p;
+    p.M = squared ? __uint_as_float(max_sq_bits) : __fsqrt_rn(__uint_as_float(max_sq_bits));
+    p.wide = !(p.M >= 1e-18f && p.M <= 1e18f);
+    p.scale = p.wide ? 0.0f : __fdiv_rn(e.inv, p.M);
+    return p;
+}
+template <int N, class Cost>
+__device__ __forceinline__ void quantise_points(const float (&sq)[N], int squared, const PointsScale &p,
+                                                const EpsSplit &e, uint32_t (&h)[N], const Cost &exact_cost) {
+    float v[N];
+    uint32_t top = 0;
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        v[j] = sq[j];
+        if (!squared) asm("sqrt.approx.f32 %0, %1;" : "=f"(v[j]) : "f"(sq[j]));
+        top = max(top, __float_as_uint(sq[j]));
+    }
+    floor_group<N>(v, p.scale, 2.0f * e.win, p.wide || top >= 0x7F800000u, h, [&](int j) {
+        const float d = squared ? sq[j] : __fsqrt_rn(sq[j]);
+        const float c = p.M > 0.0f ? __fdiv_rn(d, p.M) : 0.0f;
+        return exact_cost(d, quantise_fbits(__float_as_uint(c), e));
+    });
+}
+
+// Low bytes (16-bit halves) of four values as one stored word (pair).
+__device__ __forceinline__ uint32_t pack_bytes(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    return __byte_perm(__byte_perm(a, b, 0x0040), __byte_perm(c, d, 0x0040), 0x5410);
+}
+__device__ __forceinline__ uint32_t pack_halves(uint32_t a, uint32_t b) { return __byte_perm(a, b, 0x5410); }
+
 // Bit j of the result: 16-bit lane j of the 8-lane vector s equals t (t2 =
 // t in both halves).
 __device__ __forceinline__ unsigned eq_mask(uint4 s, uint32_t t2) {
