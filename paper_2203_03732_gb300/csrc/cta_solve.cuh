@@ -26,7 +26,7 @@
 //
 // The 512-problem batch (64 to 2048 rows, eps = 0.01) took 2.60 ms in the
 // solver with 64-bit words, past-proposal lists and a word lookup per taken
-// candidate; it takes 1.60 ms.  64 problems of 4096 points: 7.0 ms -> 1.3 ms.
+// candidate; it takes 1.52 ms.  64 problems of 4096 points: 7.0 ms -> 1.2 ms.
 // A round of few rows (n = 1000) takes about 1.5 us, of which the scan of a
 // row is 0.9 us: instructions of one warp, not its loads.  Measured and left
 // out: 4 or 8 lanes per row (the lanes' shared-memory and L1 accesses cost
@@ -48,6 +48,7 @@ static_assert(kCtaMaxCols < (1 << kCtaRowBits), "rows and resume columns must fi
 // rows per warp the same to 10 % slower.
 constexpr int kLaneSteps = 16;
 constexpr int kLaneFew = 1;
+constexpr int kLaneSure = 2;  // steps that run while any row is left
 constexpr int kLaneMin = 4;
 
 struct CtaShared {
@@ -288,7 +289,8 @@ __device__ __forceinline__ void cta_phases(CtaShared &s, const CtaState<CB> &st,
                             c += 2 * W;
                             go = a < 0 && c < ldq;
                         }
-                        if (__popc(__ballot_sync(0xFFFFFFFFu, go)) <= kLaneFew) break;
+                        const int n = __popc(__ballot_sync(0xFFFFFFFFu, go));
+                        if (n == 0 || (n <= kLaneFew && k >= kLaneSure)) break;
                     }
                     if (!later && __popc(__ballot_sync(0xFFFFFFFFu, act && a >= 0)) < 8 && lane == 0) s.far = 1;
                     // rows not settled: the whole warp scans each from where its lane stopped
@@ -308,35 +310,53 @@ __device__ __forceinline__ void cta_phases(CtaShared &s, const CtaState<CB> &st,
                         }
                     }
                     if (act) cells += a >= 0 ? (unsigned)(a - start + 1) : (start < nA ? (unsigned)(nA - start) : 0u);
-                    // proposals: lanes that share the first lane's column (losers
-                    // of one column often do) send their lowest row only
-                    int loser = -1;
+                    // proposals, all lanes together: lanes that share the first
+                    // lane's column (losers of one column often do) send their
+                    // lowest row only
+                    int loser = -1, won_a = -1, next_e = -1;
                     const unsigned has = __ballot_sync(0xFFFFFFFFu, a >= 0);
                     if (has) {
                         const int af = __shfl_sync(0xFFFFFFFFu, a, __ffs(has) - 1);
-                        const unsigned same = __ballot_sync(0xFFFFFFFFu, a == af);
+                        const unsigned low =
+                            __reduce_min_sync(0xFFFFFFFFu, a == af ? (unsigned)b : 0xFFFFFFFFu);
                         if (a >= 0) {
-                            if (a == af) {
-                                const int bm = (int)__reduce_min_sync(same, (unsigned)b);
-                                loser = b == bm ? propose(b, a) : b;
+                            if (a == af && (unsigned)b != low) {
+                                loser = b;
                             } else {
-                                loser = propose(b, a);
+                                const unsigned old = atomicMax(pw + a, Rhi | (0xFFFFu - (unsigned)b));
+                                const unsigned tag = old >> 16;
+                                const int orow = 0xFFFF - (int)(old & 0xFFFFu);
+                                if (tag == R) {
+                                    loser = max(b, orow);
+                                } else {
+                                    won_a = a;
+                                    if (tag) next_e = orow | ((a + 1) << kCtaRowBits);
+                                }
                             }
                         }
                         __syncwarp();
                     }
                     if (act && a < 0) {  // step (III b): relabel
                         y[b] += 1;
-                        lb[atomicAdd(&s.nfl[nxt], 1)] = b;
+                        next_e = b;
                     }
-                    const unsigned lost = __ballot_sync(0xFFFFFFFFu, loser >= 0);
-                    if (lost) {
-                        int base = 0;
-                        if (lane == 0) base = atomicAdd(&s.nlose[q ^ 1], __popc(lost));
-                        base = __shfl_sync(0xFFFFFFFFu, base, 0);
-                        if (loser >= 0)
-                            lose[base + __popc(lost & ((1u << lane) - 1u))] = loser | ((a + 1) << kCtaRowBits);
+                    // the three lists' places in one shared-memory trip: lane 0
+                    // takes the losers', lane 1 the won columns', lane 2 the
+                    // next phase's
+                    const unsigned m0 = __ballot_sync(0xFFFFFFFFu, loser >= 0);
+                    const unsigned m1 = __ballot_sync(0xFFFFFFFFu, won_a >= 0);
+                    const unsigned m2 = __ballot_sync(0xFFFFFFFFu, next_e >= 0);
+                    int base = 0;
+                    if (lane < 3) {
+                        int *cnt = lane == 0 ? &s.nlose[q ^ 1] : lane == 1 ? &s.nwon[pp] : &s.nfl[nxt];
+                        base = atomicAdd(cnt, __popc(lane == 0 ? m0 : lane == 1 ? m1 : m2));
                     }
+                    const unsigned below = (1u << lane) - 1u;
+                    const int b0 = __shfl_sync(0xFFFFFFFFu, base, 0), b1 = __shfl_sync(0xFFFFFFFFu, base, 1),
+                              b2 = __shfl_sync(0xFFFFFFFFu, base, 2);
+                    if (loser >= 0) lose[b0 + __popc(m0 & below)] = loser | ((a + 1) << kCtaRowBits);
+                    if (won_a >= 0) won[b1 + __popc(m1 & below)] = (uint16_t)won_a;
+                    if (next_e >= 0) lb[b2 + __popc(m2 & below)] = next_e;
                 }
             } else {
 #pragma unroll 1
