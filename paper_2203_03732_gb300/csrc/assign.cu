@@ -154,6 +154,7 @@ struct Params {
     int rule = 0;      // step I: 0 lowest-index columns, 1 seeded start columns (PR_RULE_OFFSET),
                        // 2 Israeli-Itai, 3 the sequential greedy by displacement chains
     void *ii = nullptr;  // PR_RULE_ISRAELI_ITAI's state region
+    int near = 0;  // floor(1/eps) <= kNearMaxK: later rounds' scans are short (near_scans)
     int hand = 0;  // k_phases stops at this many free rows, all in the pool, and k_solo goes on (0: never)
 };
 
@@ -590,6 +591,79 @@ __device__ __forceinline__ int warp_scan_slot(const unsigned char *slot, const C
     return -1;
 }
 
+// ---------------------------------------------------------------------------
+// Later rounds of a phase with more jobs than one register group: a row that
+// lost resumes right after its column, and at large eps (the only solves with
+// such rounds) its next candidate is near, so a row gets G lanes (8, or 16
+// while 32 jobs cover the CTA) and one 16-byte load per lane and step, at most
+// kNearSteps steps; the warp scans what is left of a row that needs more.
+// Only for floor(1/eps) <= kNearMaxK: at eps = 0.02 a later scan already
+// examines some 400 entries, and the whole solve was 0.5 % slower with it.
+// n = 10,000, eps = 0.1 (147 rounds, 30 rows per CTA, 75 entries per scan), where
+// the slots copied whole row tails: solve 1084 -> 868 us; n = 6000 634 -> 561 us,
+// n = 10,000 at eps = 0.3 7.9 -> 6.3 ms, n = 1000 (3 rows per CTA) unchanged.
+// ---------------------------------------------------------------------------
+constexpr int kNearSteps = 4;
+constexpr long long kNearMaxK = 20;
+
+template <class CB, bool F7>
+__device__ __forceinline__ void near_scans(Smem &s, const Params &p, const CB *ks, const unsigned *tk, int nq) {
+    constexpr int W = kPerLoad<CB>;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int G = nq <= 2 * kWarps ? 16 : 8, per = 32 / G, gl = lane & (G - 1);
+    unsigned long long bytes = 0;
+#pragma unroll 1
+    for (int j0 = warp * per; j0 < nq; j0 += kWarps * per) {
+        const int j = j0 + lane / G;
+        const bool act = j < nq;
+        const int start = act ? s.job_start[j] : 0, b = act ? s.job_b[j] : 0;
+        const uint32_t tgt = act ? (uint32_t)s.job_tgt[j] : 0u;
+        const uint32_t t = W == 8 ? (tgt | (tgt << 16)) : tgt * 0x01010101u;
+        const CB *row = static_cast<const CB *>(p.cb) + (size_t)b * p.ldq;
+        int c = start & ~(W - 1), a = 0x7FFFFFFF;
+        bool go = act && c < p.ldq;
+#pragma unroll 1
+        for (int k = 0; k < kNearSteps && __any_sync(0xFFFFFFFFu, go); ++k) {
+            const int idx = c + gl * W;
+            int hit = 0x7FFFFFFF;
+            if (go && idx < p.ldq) {
+                const uint4 v = ld_nc_na_v4(row + idx);
+                bytes += 16;
+                unsigned m = vec_marks<CB, F7>(v, *reinterpret_cast<const uint4 *>(ks + idx), t);
+                if (idx < start) m &= start - idx >= W ? 0u : ~0u << (start - idx);
+                m &= ~(tk[idx >> 5] >> (idx & 31));
+                if (m) hit = idx + __ffs(m) - 1;
+            }
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1)
+                if (o < G) hit = min(hit, __shfl_xor_sync(0xFFFFFFFFu, hit, o));
+            if (go) {
+                a = hit;
+                c += G * W;
+                go = a == 0x7FFFFFFF && c < p.ldq;
+            }
+        }
+        unsigned left = __ballot_sync(0xFFFFFFFFu, go && gl == 0);
+#pragma unroll 1
+        while (left) {
+            const int l = __ffs(left) - 1;
+            left &= left - 1;
+            const int bl = __shfl_sync(0xFFFFFFFFu, b, l), tl = __shfl_sync(0xFFFFFFFFu, (int)tgt, l);
+            const CB *rl = static_cast<const CB *>(p.cb) + (size_t)bl * p.ldq;
+            int al = -1, used;
+#pragma unroll 1
+            for (int c0 = __shfl_sync(0xFFFFFFFFu, c, l); c0 < p.ldq && al < 0; c0 += kChunk<CB>) {
+                al = warp_scan_chunk<CB, F7, false>(rl, ks, tk, true, c0, c0, p.ldq, p.nA, tl, nullptr, used, lane);
+                if (lane == 0) bytes += sizeof(CB) * (unsigned long long)min(kChunk<CB>, p.ldq - c0);
+            }
+            if (lane == l && al >= 0) a = al;
+        }
+        if (act && gl == 0) s.job_best[j] = a;
+    }
+    bytes = __reduce_add_sync(0xFFFFFFFFu, (unsigned)bytes);
+    if (lane == 0 && bytes) atomicAdd(&s.bytes, bytes);
+}
+
 // A bulk copy's completion wait: long enough for any copy a working GPU
 // finishes (about a second), independent of the barrier spin limit.
 constexpr long long kCopyWaitCycles = 2000000000ll;
@@ -612,11 +686,14 @@ __device__ __forceinline__ void run_jobs(Smem &s, const Lists &g, const Params &
     // slots (up to 16 rows in flight instead of rows_per_group); the choice is
     // this CTA's own.  The slot scan reads every unknown y(b) first (the
     // register scan reads it inside the row scan).
-    const bool via_slots = SL && nq > rows_per_group;
+    const bool near = !OFS && p.near && R > Rps && nq > rows_per_group;
+    const bool via_slots = SL && !near && nq > rows_per_group;
     if (via_slots)
         for (int j = threadIdx.x; j < nq; j += blockDim.x)
             if (s.job_tgt[j] < 0) s.job_tgt[j] = ld_relaxed_s32(p.y_b + s.job_b[j]) - 1;
-    if (via_slots) {
+    if (near) {
+        near_scans<CB, F7>(s, p, ks, tk, nq);
+    } else if (via_slots) {
         // warp w scans jobs w, w + nslots, ... through its own slot
         __syncthreads();
         unsigned long long my_bytes = 0;
@@ -1685,6 +1762,7 @@ pr_status launch_solve(Params &p, const CostSource &src, double eps, const Phase
     const long long K = (long long)floor(1.0 / eps);
     p.phase_cap = ((long long)n_rows * (2 * K + 3)) / (p.T + 1) + 1;
     p.spin_limit = spin_limit_cycles();
+    p.near = K <= kNearMaxK ? 1 : 0;
     p.profile = 0;
     if (profile_ok) {
         const char *pf = getenv("PR_PROFILE");
