@@ -30,12 +30,22 @@
 // One phase (B' = supply vertices with free copies), steps of k_ot_loop (one
 // cooperative launch; a grid barrier with a summed payload after each step):
 //   ot_phase_start  r_b = f_b, flags, the free-copy total for the stop test
-//   round R: ot_propose  every searching b proposes (atomicMax on the column
-//                        word) to the lowest admissible a >= its resume
-//                        column with unmatched lo copies left;
-//            ot_grant    a's lowest proposer b gets g = min(r_b, avail_a)
-//                        copies; partners of matched lo copies are evicted,
-//                        highest supply index first (step II)
+//   round R: ot_round    a b that won its column a in round R - 1 takes g =
+//                        min(r_b, avail_a) copies; partners of matched lo
+//                        copies are evicted, highest supply index first
+//                        (step II).  Then every searching b proposes
+//                        (atomicMax on the column word) to the lowest
+//                        admissible a >= its resume column with unmatched lo
+//                        copies left.
+// Grants and the next proposals share a step, so a round has one grid barrier
+// (with a step of its own for the grants, and a second barrier, a solve took
+// 1537 us at 10,000 x 10,000, eps = 0.05; now 1235 us, and 20 to 27 % less from
+// 128 x 128 to 10,000 x 3000).  A scan that meets a column granted
+// in round R - 1 must see the copies left after the grant, whether or not the
+// winner's warp has applied it yet: column words and the r_b are kept by round
+// parity, so those of round R - 1 are fixed during step R, and a column's
+// copies left carry the round of the last grant in them.  If that round is not
+// R - 1, the reader takes the winner's grant off itself.
 //   ot_phase_end    F_b += 1 for b in B' left with unplaced copies (III b);
 //                   clusters shift up where the lo cluster is empty (III a)
 // Nothing in a solve waits for the host: errors found on the device (masses,
@@ -70,7 +80,7 @@ namespace {
 
 constexpr int kOtThreads = 256;
 constexpr int kOtUnroll = 4;  // 2 KiB warp chunks (swept 3, 4, 8 at 10k x 10k)
-constexpr int kFlagSearching = 1, kFlagInBp = 2;
+constexpr int kFlagSearching = 1, kFlagStuck = 2;  // stuck: no column left, to be relabelled
 constexpr int kCostCtas = 64;  // CTAs of the cost sum (a constant: same order on every device)
 constexpr int kListSlot = 32;  // entries of a demand's first list slot (one per lane of a warp)
 
@@ -117,15 +127,15 @@ OLayout make_olayout(int nB, int nA) {
     L.D = c.take<int>(nA);
     L.F = c.take<int>(nB);
     L.f = c.take<int>(nB);
-    L.r = c.take<int>(nB);
+    L.r = c.take<int>(2 * (size_t)nB);
     L.ptr = c.take<int>(nB);
     L.flag = c.take<int>(nB);
     L.kmin = c.take<int>(nA);
     L.clo = c.take<int>(nA);
     L.chi = c.take<int>(nA);
-    L.avail = c.take<int>(nA);
+    L.avail = c.take<unsigned long long>(nA);
     L.granted = c.take<int>(nA);
-    L.prop = c.take<unsigned long long>(nA);
+    L.prop = c.take<unsigned long long>(2 * (size_t)nA);
     L.arena = ot_arena_entries(nB, nA);
     L.list_cap = (long long)nA * kListSlot + L.arena;
     L.eb = c.take<int>((size_t)L.list_cap);
@@ -159,9 +169,10 @@ struct OParams {
     OCtl *ctl;
     const void *cb;  // uint8_t or uint16_t [nB][ldq] (bytes when floor(1/eps) <= 252)
     void *key;       // k = kmin_a per column, in the same type (padding 0xFF / 0x8000)
-    int *S, *D, *F, *f, *r, *ptr, *flag;
-    int *kmin, *clo, *chi, *avail, *granted;
-    unsigned long long *prop;
+    int *S, *D, *F, *f, *r, *ptr, *flag;  // r: [2][n_sup], by round parity
+    int *kmin, *clo, *chi, *granted;
+    unsigned long long *avail;  // copies left | round of the last grant in them << 32
+    unsigned long long *prop;   // column words [2][n_dem], by round parity
     // per-demand lists: entry i of a's list is (eb, elo, ehi)[seg_off[a] + i],
     // i < seg_len[a] <= seg_cap[a]; arena slots start at n_dem * kListSlot
     int *eb, *elo, *ehi;
@@ -218,7 +229,6 @@ __global__ void k_ot_init(OParams p) {
     for (int b = t0; b < p.nB; b += stride) {
         p.F[b] = 1;
         p.f[b] = p.S[b];
-        p.r[b] = 0;
         p.ptr[b] = 0;
         p.flag[b] = 0;
     }
@@ -228,18 +238,20 @@ __global__ void k_ot_init(OParams p) {
         p.kmin[a] = 0;
         p.clo[a] = p.D[a];
         p.chi[a] = 0;
-        p.avail[a] = p.D[a];
+        p.avail[a] = (unsigned)p.D[a];
         p.granted[a] = 0;
-        p.prop[a] = word_of(0, -1);
+        p.prop[a] = p.prop[p.nA + a] = word_of(0, -1);
         p.seg_off[a] = a * kListSlot;  // every list starts empty in its first slot
         p.seg_cap[a] = kListSlot;
         p.seg_len[a] = 0;
     }
 }
 
-__global__ void k_ot_ctl_init(OCtl *c) {
-    memset(c, 0, sizeof(OCtl));
-    c->head.magic = kWsMagic;
+__global__ void k_ot_ctl_init(OCtl *c) {  // one CTA
+    static_assert(sizeof(OCtl) % 4 == 0, "cleared by words");
+    for (int i = threadIdx.x; i < (int)(sizeof(OCtl) / 4); i += blockDim.x) reinterpret_cast<unsigned *>(c)[i] = 0;
+    __syncthreads();
+    if (threadIdx.x == 0) c->head.magic = kWsMagic;
 }
 
 // Sum over the CTA of one value per thread (every thread gets the sum).
@@ -253,110 +265,23 @@ __device__ __forceinline__ unsigned long long cta_sum(unsigned long long v) {
     return acc;
 }
 
-// Phase start: r_b = f_b, B' = {b : f_b > 0}; returns this thread's free copies.
-__device__ __forceinline__ unsigned long long ot_phase_start(const OParams &p) {
+// Phase start after round R: r_b = f_b, B' = {b : f_b > 0}; returns this thread's free copies.
+__device__ __forceinline__ unsigned long long ot_phase_start(const OParams &p, unsigned R) {
+    int *r = p.r + (size_t)(R & 1) * p.nB;
     unsigned long long mine = 0;
     for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < p.nB; b += gridDim.x * blockDim.x) {
         const int fb = ld_relaxed_s32(p.f + b);  // evictions add to it from any CTA
-        p.r[b] = fb;
-        p.flag[b] = fb > 0 ? (kFlagSearching | kFlagInBp) : 0;
-        p.ptr[b] = 0;
+        r[b] = fb;
+        p.flag[b] = fb > 0 ? kFlagSearching : 0;
+        p.ptr[b] = -1;
         mine += (unsigned long long)fb;
     }
     return mine;
 }
 
-// Warp per searching supply vertex: the lowest a >= ptr with
-// cbar + kmin_a == F_b - 1 and avail_a > 0.
-// Returns this thread's proposals (lane 0 of each warp counts its rows).
-// F7: floor(1/eps) <= 125, so every sum of a real column's cbar and key
-// stays below 256 and the byte pre-test is one plain add (may_match<true>).
-template <class CB, bool F7>
-__device__ __forceinline__ unsigned ot_propose(const OParams &p, unsigned R, unsigned long long &bytes_out) {
-    constexpr int W = 16 / (int)sizeof(CB);  // columns per 16-byte load
-    constexpr unsigned kAll = W == 16 ? 0xFFFFu : 0xFFu;
-    constexpr int kChunkW = 32 * W * kOtUnroll;
-    unsigned props = 0;
-    const int lane = threadIdx.x & 31;
-    const int warp_g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    const CB *key = static_cast<const CB *>(p.key);
-    unsigned long long bytes = 0;
-    // a row's flag, dual and resume column are loaded together, and the next
-    // row's while this one is scanned (only this warp writes them in this
-    // step; other CTAs wrote them in earlier steps, so the loads go to L2)
-    int nfl = 0, nF = 0, nst = 0;
-    if (warp_g < p.nB) {
-        nfl = ld_relaxed_s32(p.flag + warp_g);
-        nF = ld_relaxed_s32(p.F + warp_g);
-        nst = ld_relaxed_s32(p.ptr + warp_g);
-    }
-    for (int b = warp_g; b < p.nB; b += nwarps) {
-        const int fl = nfl, Fb = nF, start = nst;
-        if (b + nwarps < p.nB) {
-            nfl = ld_relaxed_s32(p.flag + b + nwarps);
-            nF = ld_relaxed_s32(p.F + b + nwarps);
-            nst = ld_relaxed_s32(p.ptr + b + nwarps);
-        }
-        if (!(fl & kFlagSearching)) continue;
-        const uint32_t tgt = (uint32_t)(Fb - 1);
-        const uint32_t t2 = W == 8 ? (tgt | (tgt << 16)) : tgt * 0x01010101u;
-        const CB *row = static_cast<const CB *>(p.cb) + (size_t)b * p.ldq;
-        int found = -1;
-        for (int c0 = start & ~(W - 1); c0 < p.ldq && found < 0; c0 += kChunkW) {
-            uint4 cv[kOtUnroll];
-#pragma unroll
-            for (int u = 0; u < kOtUnroll; ++u) {
-                const int idx = c0 + u * 32 * W + lane * W;
-                cv[u] = idx < p.ldq ? ld_nc_na_v4(row + idx) : make_uint4(0, 0, 0, 0);
-            }
-            bytes += sizeof(CB) * (unsigned long long)min(kChunkW, p.ldq - c0);
-            for (int u = 0; u < kOtUnroll && found < 0; ++u) {
-                const int idx = c0 + u * 32 * W + lane * W;
-                unsigned m = 0;
-                if (idx < p.ldq) {
-                    const uint4 kv = *reinterpret_cast<const uint4 *>(key + idx);
-                    m = W == 8 ? eq_mask(make_uint4(cv[u].x + kv.x, cv[u].y + kv.y, cv[u].z + kv.z, cv[u].w + kv.w), t2)
-                               : eq_mask8<F7>(cv[u], kv, t2);
-                }
-                const int lo = start - idx;
-                if (lo > 0) m &= lo >= W ? 0u : (kAll << lo) & kAll;
-                // every lane checks its lowest candidate's copies at once;
-                // the lowest lane with copies wins once no lower lane holds
-                // a candidate (lanes are in column order)
-                for (;;) {
-                    if (__ballot_sync(0xFFFFFFFFu, m != 0) == 0) break;
-                    const int a_mine = idx + __ffs(m) - 1;
-                    const bool ok = m != 0 && ld_relaxed_s32(p.avail + a_mine) > 0;
-                    const unsigned okm = __ballot_sync(0xFFFFFFFFu, ok);
-                    if (!ok && m) m &= m - 1;
-                    if (okm) {
-                        const int L = __ffs(okm) - 1;
-                        if ((__ballot_sync(0xFFFFFFFFu, m != 0) & ((1u << L) - 1)) == 0) {
-                            found = __shfl_sync(0xFFFFFFFFu, a_mine, L);
-                            break;
-                        }
-                    }
-                }
-            }
-        }
-        if (lane == 0) {
-            if (found >= 0) {
-                atomicMax(p.prop + found, word_of(R, b));
-                p.ptr[b] = found;
-                ++props;
-            } else {
-                atomicAnd(p.flag + b, ~kFlagSearching);
-            }
-        }
-    }
-    if (lane == 0) bytes_out += bytes;
-    return props;
-}
-
 // ---------------------------------------------------------------------------
-// Per-demand lists (warp operations; only the grant or the phase end of
-// demand a touches a's list, one warp at a time)
+// Per-demand lists (warp operations; only the winner's grant or the phase end
+// of demand a touches a's list, one warp at a time)
 // ---------------------------------------------------------------------------
 // Step (II): take `need` lo copies from a's list, highest supply index first
 // (the end of the list); each copy taken rejoins its supply's free copies.
@@ -487,65 +412,144 @@ __device__ __forceinline__ void list_shift(const OParams &p, int a, int lane) {
     if (lane == 0) p.seg_len[a] = w;
 }
 
+__device__ __forceinline__ void st_relaxed_u64(unsigned long long *p, unsigned long long v) {
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+// Copies left at column a after round R - 1's grant, during step R.
+__device__ __forceinline__ int ot_left(const OParams &p, int a, unsigned R) {
+    const unsigned long long av = ld_relaxed_u64(p.avail + a);
+    const unsigned long long w = ld_relaxed_u64(p.prop + (size_t)((R - 1) & 1) * p.nA + a);
+    const int left = (int)(unsigned)av;
+    if (tag_of(w) != R - 1 || (unsigned)(av >> 32) == R - 1) return left;
+    return left - min(left, ld_relaxed_s32(p.r + (size_t)((R - 1) & 1) * p.nB + row_of(w)));
+}
+
+// Step R, a warp per searching supply vertex b.  If b won its column in round
+// R - 1, its warp applies the grant (each column has one winner, so one warp
+// touches its list and counts; f, which other grants' evictions also change,
+// changes by atomics).  If b has copies left, it proposes to the lowest a >=
+// its resume column with cbar + kmin_a == F_b - 1 and copies left.
+// Returns this thread's proposals (lane 0 of each warp counts its rows).
+// F7: floor(1/eps) <= 125, so every sum of a real column's cbar and key
+// stays below 256 and the byte pre-test is one plain add (may_match<true>).
+template <class CB, bool F7>
+__device__ __forceinline__ unsigned ot_round(const OParams &p, unsigned R, unsigned long long &bytes_out) {
+    constexpr int W = 16 / (int)sizeof(CB);  // columns per 16-byte load
+    constexpr unsigned kAll = W == 16 ? 0xFFFFu : 0xFFu;
+    constexpr int kChunkW = 32 * W * kOtUnroll;
+    unsigned props = 0;
+    const int lane = threadIdx.x & 31;
+    const int warp_g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int nwarps = (gridDim.x * blockDim.x) >> 5;
+    const CB *key = static_cast<const CB *>(p.key);
+    const int *r_old = p.r + (size_t)((R - 1) & 1) * p.nB;
+    int *r_new = p.r + (size_t)(R & 1) * p.nB;
+    const unsigned long long *words = p.prop + (size_t)((R - 1) & 1) * p.nA;
+    unsigned long long bytes = 0;
+    // a row's flag, dual, resume column and copies are loaded together, and
+    // the next row's while this one is scanned (only this warp writes them;
+    // phase starts and ends on other CTAs do too, so the loads go to L2)
+    int nfl = 0, nF = 0, nst = 0, nr = 0;
+    if (warp_g < p.nB) {
+        nfl = ld_relaxed_s32(p.flag + warp_g);
+        nF = ld_relaxed_s32(p.F + warp_g);
+        nst = ld_relaxed_s32(p.ptr + warp_g);
+        nr = ld_relaxed_s32(r_old + warp_g);
+    }
+    for (int b = warp_g; b < p.nB; b += nwarps) {
+        const int fl = nfl, Fb = nF, at = nst;
+        int rb = nr;
+        if (b + nwarps < p.nB) {
+            nfl = ld_relaxed_s32(p.flag + b + nwarps);
+            nF = ld_relaxed_s32(p.F + b + nwarps);
+            nst = ld_relaxed_s32(p.ptr + b + nwarps);
+            nr = ld_relaxed_s32(r_old + b + nwarps);
+        }
+        if (!(fl & kFlagSearching)) continue;
+        int g = 0, km = 0;  // copies granted to b at column `at`, and its kmin
+        if (at >= 0 && ld_relaxed_u64(words + at) == word_of(R - 1, b)) {
+            const int left = (int)(unsigned)ld_relaxed_u64(p.avail + at);
+            km = p.kmin[at];
+            g = min(rb, left);
+            rb -= g;
+            if (lane == 0) {
+                st_relaxed_u64(p.avail + at, ((unsigned long long)(R - 1) << 32) | (unsigned)(left - g));
+                p.clo[at] -= g;
+                p.chi[at] += g;
+                p.granted[at] = 1;
+                atomicSub(p.f + b, g);
+            }
+            __syncwarp();
+        }
+        int found = -1;
+        if (rb > 0) {
+            const int start = at > 0 ? at : 0;
+            const uint32_t tgt = (uint32_t)(Fb - 1);
+            const uint32_t t2 = W == 8 ? (tgt | (tgt << 16)) : tgt * 0x01010101u;
+            const CB *row = static_cast<const CB *>(p.cb) + (size_t)b * p.ldq;
+            for (int c0 = start & ~(W - 1); c0 < p.ldq && found < 0; c0 += kChunkW) {
+                uint4 cv[kOtUnroll];
+#pragma unroll
+                for (int u = 0; u < kOtUnroll; ++u) {
+                    const int idx = c0 + u * 32 * W + lane * W;
+                    cv[u] = idx < p.ldq ? ld_nc_na_v4(row + idx) : make_uint4(0, 0, 0, 0);
+                }
+                bytes += sizeof(CB) * (unsigned long long)min(kChunkW, p.ldq - c0);
+                for (int u = 0; u < kOtUnroll && found < 0; ++u) {
+                    const int idx = c0 + u * 32 * W + lane * W;
+                    unsigned m = 0;
+                    if (idx < p.ldq) {
+                        const uint4 kv = *reinterpret_cast<const uint4 *>(key + idx);
+                        m = W == 8 ? eq_mask(make_uint4(cv[u].x + kv.x, cv[u].y + kv.y, cv[u].z + kv.z, cv[u].w + kv.w), t2)
+                                   : eq_mask8<F7>(cv[u], kv, t2);
+                    }
+                    const int lo = start - idx;
+                    if (lo > 0) m &= lo >= W ? 0u : (kAll << lo) & kAll;
+                    // every lane checks its lowest candidate's copies at once;
+                    // the lowest lane with copies wins once no lower lane holds
+                    // a candidate (lanes are in column order)
+                    for (;;) {
+                        if (__ballot_sync(0xFFFFFFFFu, m != 0) == 0) break;
+                        const int a_mine = idx + __ffs(m) - 1;
+                        const bool ok = m != 0 && ot_left(p, a_mine, R) > 0;
+                        const unsigned okm = __ballot_sync(0xFFFFFFFFu, ok);
+                        if (!ok && m) m &= m - 1;
+                        if (okm) {
+                            const int L = __ffs(okm) - 1;
+                            if ((__ballot_sync(0xFFFFFFFFu, m != 0) & ((1u << L) - 1)) == 0) {
+                                found = __shfl_sync(0xFFFFFFFFu, a_mine, L);
+                                break;
+                            }
+                        }
+                    }
+                }
+            }
+        }
+        if (lane == 0) {
+            if (found >= 0) {
+                atomicMax(p.prop + (size_t)(R & 1) * p.nA + found, word_of(R, b));
+                p.ptr[b] = found;
+                r_new[b] = rb;
+                ++props;
+            } else {
+                p.flag[b] = rb > 0 ? kFlagStuck : 0;
+            }
+        }
+        if (g > 0) {
+            if (km >= 1) list_evict(p, at, g, lane);
+            __syncwarp();
+            list_add_hi(p, at, b, g, lane);
+        }
+    }
+    if (lane == 0) bytes_out += bytes;
+    return props;
+}
+
 // The demands of one wave of the grid, CTA-minor: thread t of CTA c takes
 // demand c + t * G, so every CTA gets about n_dem / G of them.
 __device__ __forceinline__ int wave_demand(int base, unsigned G) {
     return base + (int)(threadIdx.x * G + blockIdx.x);
-}
-
-// Grant step: thread per demand a that received a proposal in round R; its
-// lowest proposer b takes g = min(r_b, avail_a) copies.  The grants go on a
-// CTA list; after a CTA barrier each warp takes one listed grant: if a's
-// copies are matched (kmin_a >= 1) it evicts g of them (step II), then it
-// adds b's g copies to a's list.  Every a has one winner and touches only its
-// own list, and the counts other grants also touch (f) change by atomics, so
-// the order of the grants does not matter.
-__device__ __forceinline__ void ot_grant(const OParams &p, unsigned R) {
-    __shared__ int gl_a[kOtThreads], gl_b[kOtThreads], gl_g[kOtThreads];
-    __shared__ int n_gl;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const unsigned G = gridDim.x;
-    for (int base = 0; base < p.nA; base += (int)(G * blockDim.x)) {
-        if (threadIdx.x == 0) n_gl = 0;
-        __syncthreads();
-        const int a = wave_demand(base, G);
-        if (a < p.nA) {
-            // the column's word and the winner's remaining copies were written
-            // by other CTAs: coherent loads (L2), never a line this SM's L1
-            // kept from an earlier round
-            const unsigned long long w = ld_relaxed_u64(p.prop + a);
-            if (tag_of(w) == R) {
-                const int b = row_of(w);
-                // the values a winner needs, loaded at once (only a's winner
-                // writes them in this step)
-                const int av = p.avail[a];
-                const int rb = ld_relaxed_s32(p.r + b);
-                const int km = p.kmin[a];
-                const int g = rb < av ? rb : av;
-                p.avail[a] = av - g;
-                p.r[b] = rb - g;
-                if (rb - g == 0) atomicAnd(p.flag + b, ~kFlagSearching);
-                p.clo[a] -= g;
-                p.chi[a] += g;
-                p.granted[a] = 1;
-                atomicSub(p.f + b, g);
-                if (g > 0) {
-                    const int k = atomicAdd(&n_gl, 1);
-                    gl_a[k] = a;
-                    gl_b[k] = b;
-                    gl_g[k] = km >= 1 ? -g : g;  // negative: matched copies are taken
-                }
-            }
-        }
-        __syncthreads();
-        for (int e = warp; e < n_gl; e += nw) {
-            const int ga = gl_a[e], gg = gl_g[e];
-            if (gg < 0) list_evict(p, ga, -gg, lane);
-            __syncwarp();
-            list_add_hi(p, ga, gl_b[e], gg < 0 ? -gg : gg, lane);
-        }
-        __syncthreads();
-    }
 }
 
 template <class CB>
@@ -557,7 +561,7 @@ __device__ __forceinline__ void ot_phase_end(const OParams &p) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const unsigned G = gridDim.x;
     for (int b = t0; b < p.nB; b += stride)
-        if ((ld_relaxed_s32(p.flag + b) & kFlagInBp) && ld_relaxed_s32(p.r + b) > 0) p.F[b] += 1;  // step (III b)
+        if (ld_relaxed_s32(p.flag + b) & kFlagStuck) p.F[b] += 1;  // step (III b)
     for (int base = 0; base < p.nA; base += (int)(G * blockDim.x)) {
         if (threadIdx.x == 0) n_sh = 0;
         __syncthreads();
@@ -572,7 +576,7 @@ __device__ __forceinline__ void ot_phase_end(const OParams &p) {
                 p.chi[a] = 0;
                 sh_a[atomicAdd(&n_sh, 1)] = a;
             }
-            p.avail[a] = p.clo[a];
+            p.avail[a] = (unsigned)p.clo[a];
         }
         __syncthreads();
         for (int e = warp; e < n_sh; e += nw) list_shift(p, sh_a[e], lane);
@@ -608,7 +612,7 @@ __global__ void __launch_bounds__(kOtThreads, 4) k_ot_loop(OParams p, double eps
     unsigned R = 0;
     unsigned long long bytes = 0;
     for (;;) {
-        const unsigned long long nf = cta_sum(ot_phase_start(p));
+        const unsigned long long nf = cta_sum(ot_phase_start(p, R));
         if (!grid_sum_barrier(c->bar, &c->head, gen, G, spin_limit, nf, sum)) return;
         const long long nfree = (long long)sum;
         if (nfree <= T || phases >= cap) {
@@ -631,12 +635,10 @@ __global__ void __launch_bounds__(kOtThreads, 4) k_ot_loop(OParams p, double eps
                 if (blockIdx.x == 0 && threadIdx.x == 0) record_error(&c->head, PR_ERR_INTERNAL);
                 return;
             }
-            const unsigned long long np = cta_sum(ot_propose<CB, F7>(p, R, bytes));
+            const unsigned long long np = cta_sum(ot_round<CB, F7>(p, R, bytes));
             if (!grid_sum_barrier(c->bar, &c->head, gen, G, spin_limit, np, sum)) return;
-            if (sum == 0) break;
+            if (sum == 0) break;  // and every grant has been applied
             ++rounds;
-            ot_grant(p, R);
-            if (!grid_sum_barrier(c->bar, &c->head, gen, G, spin_limit, 0, sum)) return;
         }
         ot_phase_end<CB>(p);
         if (!grid_sum_barrier(c->bar, &c->head, gen, G, spin_limit, 0, sum)) return;
@@ -1129,7 +1131,7 @@ extern "C" pr_status pr_ot(const void *C, pr_dtype dt, int64_t ldc, int32_t n_su
     p.kmin = (int *)(w + L.kmin);
     p.clo = (int *)(w + L.clo);
     p.chi = (int *)(w + L.chi);
-    p.avail = (int *)(w + L.avail);
+    p.avail = (unsigned long long *)(w + L.avail);
     p.granted = (int *)(w + L.granted);
     p.prop = (unsigned long long *)(w + L.prop);
     p.eb = (int *)(w + L.eb);
@@ -1145,7 +1147,7 @@ extern "C" pr_status pr_ot(const void *C, pr_dtype dt, int64_t ldc, int32_t n_su
 
     const DeviceInfo &di = device_info();
     const int g1 = di.sms * 4;
-    k_ot_ctl_init<<<1, 1, 0, st>>>(p.ctl);
+    k_ot_ctl_init<<<1, 256, 0, st>>>(p.ctl);
     PR_CUDA(cudaGetLastError());
     k_ot_counts<<<g1, 256, 0, st>>>(supply, demand, nB, nA, theta, p.S, p.D, p.ctl);
     PR_CUDA(cudaGetLastError());
