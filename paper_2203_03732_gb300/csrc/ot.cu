@@ -1186,7 +1186,10 @@ extern "C" pr_status pr_ot(const void *C, pr_dtype dt, int64_t ldc, int32_t n_su
         int per_sm = 0;
         PR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, loop, kOtThreads, 0));
         if (per_sm < 1) return fail(PR_ERR_INVALID, "pr_ot: loop kernel does not fit on an SM");
-        const int grid = std::min(di.sms * per_sm, 1023);
+        // no more CTAs than there are supply rows for their warps (or demands
+        // for their threads): idle CTAs only make the barriers dearer
+        const int want = std::max((nB + kOtThreads / 32 - 1) / (kOtThreads / 32), (nA + kOtThreads - 1) / kOtThreads);
+        const int grid = std::min(std::min(di.sms * per_sm, 1023), want);
         const long long limit = spin_limit_cycles();
         void *args[] = {(void *)&p, (void *)&eps, (void *)&limit};
         PR_CUDA(cudaLaunchCooperativeKernel(loop, dim3(grid), dim3(kOtThreads), args, 0, st));
