@@ -71,6 +71,7 @@ constexpr int kListSm = 1024;             // proposal-list entries kept in share
 constexpr int kKeepMax = 16;              // rows a CTA may keep for its next phase
 constexpr int kBatch = 256;               // items turned into scan jobs at a time
 constexpr int kMaxGrid = 1023;            // barrier payload field width
+constexpr unsigned kMidRounds = 16;       // rounds of a phase before k_solo may take over inside it
 
 // Control block at the start of the workspace.
 struct Ctl {
@@ -99,6 +100,9 @@ struct Ctl {
     unsigned long long prof_slot[2][8];  // per round parity: max over CTAs
     unsigned long long prof_rounds;
     unsigned long long seq_tail;  // PR_RULE_SEQUENTIAL: rows queued so far (rule_seq.cuh)
+    unsigned long long hand_start;  // and, at a take-over, the first of them that is still to run
+    int mid_rows;      // take-over inside a phase: rows that lost the last round (in p.lists)
+    unsigned mid_rps;  // ... and the phase's first round
 };
 constexpr int kProfSegs = 7;
 
@@ -155,6 +159,7 @@ struct Params {
                        // 2 Israeli-Itai, 3 the sequential greedy by displacement chains
     void *ii = nullptr;  // PR_RULE_ISRAELI_ITAI's state region
     int near = 0;  // floor(1/eps) <= kNearMaxK: later rounds' scans are short (near_scans)
+    int mid = 0;   // k_phases stops inside a phase of kMidRounds rounds, and k_solo goes on
     int hand = 0;  // k_phases stops at this many free rows, all in the pool, and k_solo goes on (0: never)
 };
 
@@ -888,7 +893,7 @@ k_phases(Params p, int warps_per_row, int rows_per_group) {
     // With at most two rows per register group (long rows) every free row
     // goes to the pool, which deals them out evenly (measured at n = 10,000:
     // 1-3 % faster than keeping one); shorter rows keep up to a group's worth.
-    const int keep = rows_per_group > 2 && p.hand == 0 ? min(rows_per_group - 1, kKeepMax) : 0;
+    const int keep = rows_per_group > 2 && p.hand == 0 && p.mid == 0 ? min(rows_per_group - 1, kKeepMax) : 0;
     // Every next-phase row goes to the pool and no CTA takes more than kBatch
     // rows in a round (so its donations of a round fit s.don): the barrier
     // places the donations (grid_sync_pool).
@@ -1123,6 +1128,20 @@ k_phases(Params p, int warps_per_row, int rows_per_group) {
             first_round = false;
             qcur ^= 1;
             if (!((pub >> 30) & 1ull)) break;  // no contested column: phase over
+            if (p.mid && R - Rps + 1 >= kMidRounds) {
+                // the rows that lost this round, for k_solo (the list written
+                // in this round is qcur ^ 1 by now)
+                for (int i = threadIdx.x; i < s.nql[qcur ^ 1]; i += blockDim.x) {
+                    const int4 q = ql_get(s, g, qcur ^ 1, i);
+                    if (row_of(ld_relaxed_u64(p.prop + q.y)) != q.x)
+                        p.lists[atomicAdd(&ctl->mid_rows, 1)] = q.x | ((q.y + 1) << kCtaRowBits);
+                }
+                if (cta == 0 && threadIdx.x == 0) {
+                    ctl->free_at_stop = (int)nf_next;  // queued for the next phase so far
+                    ctl->mid_rps = Rps;
+                }
+                goto done;
+            }
         }
         ++phase;
         if (threadIdx.x == 0) s.nfl[cur] = 0;
@@ -1281,11 +1300,25 @@ __global__ void k_solo_init(Ctl *c) {
     c->head.magic = kWsMagic;
 }
 
-// RESUME: the first phases ran in k_phases, which stopped at hand_rows free
-// rows: the state is taken over from its words, keys, duals and row pool.
-template <class CB, bool F7, bool RESUME, class Src>
+// The matched costs that k_solo adds up, whatever their source.
+struct SoloCost {
+    const void *C;
+    long long ldc;
+    int f64;
+    PointsCost pts;  // used when C is null
+    __device__ double operator()(int b, int a) const {
+        if (!C) return pts(b, a);
+        return f64 ? static_cast<const double *>(C)[(long long)b * ldc + a]
+                   : (double)static_cast<const float *>(C)[(long long)b * ldc + a];
+    }
+};
+
+// RESUME: the first phases ran in k_phases (SEQ: k_seq), which stopped at a
+// few free rows or inside a phase: the state is taken over from its words,
+// keys, duals and row lists.
+template <class CB, bool F7, bool RESUME, bool SEQ>
 __global__ void __launch_bounds__(kSoloThreads)
-k_solo(Params p, Src src, int *match_b, int *match_a, int *y_col, double *cost) {
+k_solo(Params p, SoloCost src, int *match_b, int *match_a, int *y_col, double *cost) {
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ CtaShared s;
     __shared__ double part[kFinThreads];
@@ -1294,32 +1327,58 @@ k_solo(Params p, Src src, int *match_b, int *match_a, int *y_col, double *cost) 
     const CtaLayout L(p.nB, p.nA);
     const CtaState<CB> st(dyn, L);
     CtaCounts c = {0, 0, 0, 0, false};
-    int nf = p.nB;
+    int nf = p.nB, mid = 0;
     if (RESUME) {
         c.phases = ctl->phases;
         c.rounds = ctl->rounds;
         c.barriers = (long long)ctl->barriers;
         nf = ctl->free_at_stop;
+        mid = SEQ ? 0 : ctl->mid_rows;
+        cta_begin(s, st, p.ldq, nf);
+        __syncthreads();
         for (int a = threadIdx.x; a < p.ldq; a += blockDim.x) {
-            const unsigned k = p.ka[a];
-            st.ks[a] = sizeof(CB) == 1 && k > 0xFFu ? (CB)0xFF : (CB)k;
+            unsigned k = p.ka[a];
             if (a < p.nA) {
                 const unsigned long long w = p.prop[a];
                 st.pw[a] = tag_of(w) > 0 ? 0x10000u | (0xFFFFu - (unsigned)row_of(w)) : 0u;
+                if (mid > 0 && tag_of(w) >= ctl->mid_rps) {  // won in the unfinished phase: its key rises at the end
+                    --k;
+                    atomicOr(st.tk + (a >> 5), 1u << (a & 31));
+                    st.won[atomicAdd(&s.nwon[(c.phases + 1) & 1], 1)] = (uint16_t)a;
+                }
             }
+            st.ks[a] = sizeof(CB) == 1 && k > 0xFFu ? (CB)0xFF : (CB)k;
         }
         for (int b = threadIdx.x; b < p.nB; b += blockDim.x) st.y[b] = (uint16_t)p.y_b[b];
-        const int2 *pool = p.pool + (size_t)(c.phases & 1) * p.nB;
-        if (nf > p.T)
-            for (int i = threadIdx.x; i < nf; i += blockDim.x) {
-                const int2 e = pool[i];
-                st.la[i] = e.x | ((e.y < 0 ? -1 - e.y : 0) << kCtaRowBits);
+        if (SEQ) {
+            const int4 *ring = reinterpret_cast<const int4 *>(p.lists);
+            if (nf > p.T)
+                for (int i = threadIdx.x; i < nf; i += blockDim.x) {
+                    const int4 e = ring[(ctl->hand_start + i) % (2ull * (unsigned long long)p.nB)];
+                    st.la[i] = e.x | (e.y << kCtaRowBits);
+                }
+        } else {
+            // the queued rows are in the pool of the phase that follows
+            const int2 *pool = p.pool + (size_t)((c.phases + (mid > 0)) & 1) * p.nB;
+            int *to = mid > 0 ? st.lb : st.la;
+            if (mid > 0 || nf > p.T)
+                for (int i = threadIdx.x; i < nf; i += blockDim.x) {
+                    const int2 e = pool[i];
+                    to[i] = e.x | ((e.y < 0 ? -1 - e.y : 0) << kCtaRowBits);
+                }
+            for (int i = threadIdx.x; i < mid; i += blockDim.x) st.la[i] = p.lists[i];
+            if (mid > 0 && threadIdx.x == 0) {
+                s.nfl[0] = mid;
+                s.nfl[1] = nf;
             }
+        }
     } else {
         cta_init(s, st, p.nB, p.nA, p.ldq);
     }
-    cta_phases<4, CB, F7, true>(s, st, static_cast<const CB *>(p.cb), p.nB, p.nA, p.ldq, p.T, p.phase_cap,
-                                RESUME ? 1u : 0u, nf, c);
+    __syncthreads();
+    const CB *cb = static_cast<const CB *>(p.cb);
+    if (SEQ) cta_seq_phases<4, CB, F7>(s, st, cb, p.nA, p.ldq, p.T, p.phase_cap, RESUME ? 1u : 0u, nf, c);
+    else cta_phases<4, CB, F7, true>(s, st, cb, p.nB, p.nA, p.ldq, p.T, p.phase_cap, RESUME ? 1u : 0u, nf, mid, c);
     if (threadIdx.x == 0) {
         ctl->phases = c.phases;
         ctl->rounds = c.rounds;
@@ -1334,13 +1393,13 @@ k_solo(Params p, Src src, int *match_b, int *match_a, int *y_col, double *cost) 
     cta_finish<CB>(s, dyn, L, p.nB, p.nA, part, kFinThreads, src, match_b, match_a, p.y_b, y_col, cost);
 }
 
-template <bool RESUME, class Src>
-pr_status launch_solo(const Params &p, const Src &src, bool cb8, bool f7, int *match_b, int *match_a, int *y_col,
+template <bool RESUME, bool SEQ>
+pr_status launch_solo(const Params &p, const SoloCost &src, bool cb8, bool f7, int *match_b, int *match_a, int *y_col,
                       double *cost, cudaStream_t st) {
     const size_t smem = CtaLayout(p.nB, p.nA).total(cb8 ? 1 : 2);
-    const auto fn = !cb8 ? k_solo<uint16_t, false, RESUME, Src>
-                    : f7 ? k_solo<uint8_t, true, RESUME, Src>
-                         : k_solo<uint8_t, false, RESUME, Src>;
+    const auto fn = !cb8 ? k_solo<uint16_t, false, RESUME, SEQ>
+                    : f7 ? k_solo<uint8_t, true, RESUME, SEQ>
+                         : k_solo<uint8_t, false, RESUME, SEQ>;
     // one value for every size, so that calls from several threads agree
     const int smem_max = (int)((size_t)device_info().max_smem_optin - kCtaStaticSmem);
     PR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
@@ -1620,23 +1679,39 @@ bool use_cluster(const PhaseCfg &cfg, int nslots, int n_rows, long long K, int r
 // 6000 in 16 bits: 43.0 against 41.8).
 constexpr int kSoloMaxRows = 384;
 constexpr int kHandRows = 64, kHandBytes = 256 * 1024, kHandRowBytes = 8192;
+// At floor(1/eps) <= kNearMaxK most of a solve can be one phase of a hundred
+// rounds in which hundreds of rows lose the same columns (squared distances, n
+// = 1000, eps = 0.1: 131 rounds of 464 rows).  The grid's rounds cost 4.3 us,
+// one CTA's 2.3 us at 512 to 1024 rows, so one CTA takes over inside a phase
+// that has lasted kMidRounds rounds: that solve 574 -> 347 us, n = 1500 855 -> 552
+// us, n = 1000 at eps = 0.3 1545 -> 701 us.  (A problem of 20 rounds is faster on
+// the grid: n = 1000, Euclidean, 122 us against 153 us on one CTA; at n = 2000
+// such a problem is 8 % slower with the take-over, 228 against 210 us.)
+constexpr int kMidRows = 1536;
 
-// Whether one CTA runs the problem from the start (solo), or takes over from
-// the grid once at most `hand` rows are free (0: never).
-void use_cta(const Params &p, size_t smem_max, int key_bytes, bool &solo, int &hand) {
+// Whether one CTA runs the problem from the start (solo), takes over from the
+// grid once at most p.hand rows are free (0: never), or inside a long phase
+// (p.mid).
+void use_cta(Params &p, size_t smem_max, int key_bytes, long long K, bool &solo) {
     solo = false;
-    hand = 0;
-    if (p.rule != PR_RULE_LOWEST || p.profile || p.nA > kCtaMaxCols) return;
+    p.hand = p.mid = 0;
+    if ((p.rule != PR_RULE_LOWEST && p.rule != PR_RULE_SEQUENTIAL) || p.profile || p.nA > kCtaMaxCols) return;
     if (CtaLayout(p.nB, p.nA).total(key_bytes) + kCtaStaticSmem > smem_max) return;
     const char *m = getenv("PR_PHASE_MODE");
     if (m && (strcmp(m, "grid") == 0 || strcmp(m, "cluster") == 0)) return;
-    if (m ? strcmp(m, "solo") == 0 : p.nB <= kSoloMaxRows) {
+    const bool seq = p.rule == PR_RULE_SEQUENTIAL;
+    if (m ? strcmp(m, "solo") == 0 : p.nB <= kSoloMaxRows && !seq) {
         solo = true;
         return;
     }
+    // the sequential rule: half the bytes, and never from the start (ms, grid /
+    // take-over: n = 200, eps = 0.01 2.28 / 0.63, n = 1000, eps = 0.003 24.1 /
+    // 9.0, n = 2000, eps = 0.01 1.85 / 1.43; n = 4000, eps = 0.01 with 64 rows of
+    // 4 KB 2.10 / 2.26; n = 384, eps = 0.1 on one CTA alone 0.07 / 0.17)
     const int row_bytes = p.ldq * key_bytes;
-    const int rows = std::min(kHandRows, kHandBytes / row_bytes);
-    if (row_bytes <= kHandRowBytes && rows > p.T) hand = rows;
+    const int rows = std::min(kHandRows, (seq ? kHandBytes / 2 : kHandBytes) / row_bytes);
+    if (row_bytes <= kHandRowBytes && rows > p.T) p.hand = rows;
+    p.mid = !seq && K <= kNearMaxK && p.nB <= kMidRows;
 }
 
 // Row scans of the grid form: a CTA with more jobs than one register group
@@ -1773,7 +1848,8 @@ pr_status launch_solve(Params &p, const CostSource &src, double eps, const Phase
 
     const DeviceInfo &di = device_info();
     bool solo;
-    use_cta(p, cfg.smem, cb8 ? 1 : 2, solo, p.hand);
+    use_cta(p, cfg.smem, cb8 ? 1 : 2, K, solo);
+    const bool take_over = p.hand > 0 || p.mid != 0;
     if (solo) k_solo_init<<<1, 1, 0, st>>>(p.ctl);
     else k_init<<<di.sms * 2, 256, 0, st>>>(p, row_to_col);
     PR_CUDA(cudaGetLastError());
@@ -1815,7 +1891,7 @@ pr_status launch_solve(Params &p, const CostSource &src, double eps, const Phase
     const int kb = cb8 ? 1 : 2;  // bytes per key in the shared-memory copy
     const size_t slot_room = cfg.smem > slots_offset(p.ldq, kb) ? cfg.smem - slots_offset(p.ldq, kb) : 0;
     p.nslots = (int)std::min<size_t>((size_t)kWarps, slot_room / (size_t)p.slot_bytes);
-    const bool cluster = !solo && p.hand == 0 && p.rule <= PR_RULE_OFFSET && use_cluster(cfg, p.nslots, n_rows, K, p.rule);
+    const bool cluster = !solo && !take_over && p.rule <= PR_RULE_OFFSET && use_cluster(cfg, p.nslots, n_rows, K, p.rule);
     if (solo) {
         // below
     } else if (p.rule == PR_RULE_SEQUENTIAL) {
@@ -1872,24 +1948,23 @@ pr_status launch_solve(Params &p, const CostSource &src, double eps, const Phase
         const size_t smem = sl ? slots_offset(p.ldq, kb) + (size_t)p.nslots * p.slot_bytes : smem_bytes(p.ldq, kb);
         PR_CUDA(cudaLaunchCooperativeKernel(fn, dim3(cfg.grid), dim3(kThreads), args, smem, st));
     }
-    if (solo || p.hand) {
-        const auto run = [&](auto cost_src) {
-            return solo ? launch_solo<false>(p, cost_src, cb8, f7, row_to_col, col_to_row, y_col, cost, st)
-                        : launch_solo<true>(p, cost_src, cb8, f7, row_to_col, col_to_row, y_col, cost, st);
-        };
-        const pr_status rc = src.points     ? run(PointsCost{src.XA, src.XB, src.dim, src.squared})
-                             : dt == PR_F64 ? run(MatrixCost<double>{(const double *)C, ldc})
-                                            : run(MatrixCost<float>{(const float *)C, ldc});
+    if (solo || take_over) {
+        const SoloCost cost_src{src.points ? nullptr : C, ldc, dt == PR_F64,
+                                PointsCost{src.XA, src.XB, src.dim, src.squared}};
+        const bool seq = p.rule == PR_RULE_SEQUENTIAL;
+        const auto launch = solo ? (seq ? launch_solo<false, true> : launch_solo<false, false>)
+                                 : (seq ? launch_solo<true, true> : launch_solo<true, false>);
+        const pr_status rc = launch(p, cost_src, cb8, f7, row_to_col, col_to_row, y_col, cost, st);
         if (rc != PR_OK) return rc;
     }
     if (ev0 && ev1) PR_CUDA(cudaEventRecord(ev1, st));
 
-    if (!solo && !p.hand) k_decode<<<di.sms * 2, 256, 0, st>>>(p, row_to_col, col_to_row, y_col);
+    if (!solo && !take_over) k_decode<<<di.sms * 2, 256, 0, st>>>(p, row_to_col, col_to_row, y_col);
     PR_CUDA(cudaGetLastError());
     // completion scratch: the first CTA's list region (free after the loop)
     int *free_b = p.lists;
     int *free_a = p.lists + n_rows;
-    if (solo || p.hand) {
+    if (solo || take_over) {
         // done by k_solo
     } else if (src.points)
         k_finish<PointsCost><<<1, kFinThreads, 0, st>>>(p, PointsCost{src.XA, src.XB, src.dim, src.squared},

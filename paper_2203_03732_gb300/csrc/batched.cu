@@ -318,7 +318,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_bsolve(BParams p) {
         const CB *cb = static_cast<const CB *>(p.cb) + D.cb_off;
         CtaCounts c = {0, 0, 0, 0, false};
         cta_init(s, state, D.n, D.n, D.ldq);
-        cta_phases<UNROLL, CB, F7, false>(s, state, cb, D.n, D.n, D.ldq, D.T, D.cap, 0u, D.n, c);
+        __syncthreads();
+        cta_phases<UNROLL, CB, F7, false>(s, state, cb, D.n, D.n, D.ldq, D.T, D.cap, 0u, D.n, 0, c);
         my_phases += c.phases;
         my_rounds += c.rounds;
         if (threadIdx.x == 0) {

@@ -186,9 +186,24 @@ struct CtaState {
           tk(reinterpret_cast<unsigned *>(dyn + L.taken((int)sizeof(CB)))) {}
 };
 
+// Counters at the start of cta_phases or cta_seq_phases, the first list
+// holding nf rows; the taken set empty.  Barrier before and after by the
+// caller.
+template <class CB>
+__device__ __forceinline__ void cta_begin(CtaShared &s, const CtaState<CB> &c, int ldq, int nf) {
+    for (int w = threadIdx.x; w < (ldq + 31) / 32; w += blockDim.x) c.tk[w] = 0;
+    if (threadIdx.x == 0) {
+        s.nfl[0] = nf;
+        s.nfl[1] = s.nlose[0] = s.nlose[1] = s.nwon[0] = s.nwon[1] = 0;
+        s.far = 0;
+        s.bytes = s.rows = s.cells = 0;
+    }
+}
+
 // Initialisation of a solve (Sec. 2.2): y(b) = eps, y(a) = 0, M empty, B' = B.
 template <class CB>
 __device__ __forceinline__ void cta_init(CtaShared &s, const CtaState<CB> &c, int nB, int nA, int ldq) {
+    cta_begin(s, c, ldq, nB);
     for (int a = threadIdx.x; a < ldq; a += blockDim.x) c.ks[a] = a < nA ? (CB)0 : (CB)(sizeof(CB) == 1 ? 0xFF : kPadKey);
     for (int a = threadIdx.x; a < nA; a += blockDim.x) c.pw[a] = 0;  // round 0: never won
     for (int b = threadIdx.x; b < nB; b += blockDim.x) {
@@ -198,11 +213,14 @@ __device__ __forceinline__ void cta_init(CtaShared &s, const CtaState<CB> &c, in
 }
 
 // Runs the phases from `nf` rows in the first list and round tags up to
-// `R`; `out` carries the counts on.  On return the words, row duals and keys
-// hold the result.  Every thread of the CTA calls it.
+// `R`; `out` carries the counts on.  With mid > 0 it goes on inside a phase
+// whose next round has the `mid` rows of the first list: the taken set, the
+// won columns and the next phase's list (and their counters) hold that
+// phase's so far.  On return the words, row duals and keys hold the result.
+// Every thread of the CTA calls it, after a barrier.
 template <int UNROLL, class CB, bool F7, bool KEEP>
 __device__ __forceinline__ void cta_phases(CtaShared &s, const CtaState<CB> &st, const CB *__restrict__ cb, int nB,
-                                           int nA, int ldq, int T, long long cap, unsigned R, int nf, CtaCounts &out) {
+                                           int nA, int ldq, int T, long long cap, unsigned R, int nf, int mid, CtaCounts &out) {
     constexpr int W = 16 / (int)sizeof(CB);
     unsigned *const pw = st.pw, *const tk = st.tk;
     int *la = st.la, *lb = st.lb, *const lq = st.lq;
@@ -211,23 +229,14 @@ __device__ __forceinline__ void cta_phases(CtaShared &s, const CtaState<CB> &st,
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int lane = tid & 31, warp = tid >> 5, nwarps = nthr >> 5;
 
-    for (int w = tid; w < (ldq + 31) / 32; w += nthr) tk[w] = 0;
-    if (tid == 0) {
-        s.nfl[0] = nf;
-        s.nfl[1] = s.nlose[0] = s.nlose[1] = s.nwon[0] = s.nwon[1] = 0;
-        s.far = 0;
-        s.bytes = s.rows = s.cells = 0;
-    }
-    __syncthreads();
-
     int cur = 0;
     bool near = true;  // the same in every thread: read between a round's two barriers
     bool loaded = false;  // cv holds the first chunk of entry e0, this warp's first row of the round
     int e0 = 0;
     uint4 cv[UNROLL];
     unsigned long long my_cells = 0, my_rows = 0, my_bytes = 0;
-    while (nf > T) {
-        if (out.phases >= cap) {
+    while (mid > 0 || nf > T) {
+        if (mid == 0 && out.phases >= cap) {
             out.failed = true;
             break;
         }
@@ -239,9 +248,13 @@ __device__ __forceinline__ void cta_phases(CtaShared &s, const CtaState<CB> &st,
             R = 1;
             __syncthreads();
         }
-        const unsigned Rps = R + 1;
+        const unsigned Rps = mid ? R : R + 1;
         const int pp = (int)(out.phases & 1), nxt = cur ^ 1;
-        int items = nf, nwon_seen = 0, q = 0;
+        int items = mid ? mid : nf, nwon_seen = mid ? s.nwon[pp] : 0, q = 0;
+        if (mid) {
+            mid = 0;
+            __syncthreads();  // every thread has read the won count
+        }
         const int *in = la;
         int *lose = lq;
         for (;;) {
@@ -450,6 +463,107 @@ __device__ __forceinline__ void cta_phases(CtaShared &s, const CtaState<CB> &st,
     if (my_cells) atomicAdd(&s.cells, my_cells);
     if (my_bytes) atomicAdd(&s.bytes, my_bytes);
     if (my_rows) atomicAdd(&s.rows, my_rows);
+    __syncthreads();
+}
+
+// The same with the sequential greedy as step (I) (rule_seq.cuh: chains on
+// phase-tagged words; the result does not depend on their order).  A warp per
+// row; `ph` is the tag of the last phase run.
+template <int UNROLL, class CB, bool F7>
+__device__ __forceinline__ void cta_seq_phases(CtaShared &s, const CtaState<CB> &st, const CB *__restrict__ cb, int nA,
+                                               int ldq, int T, long long cap, unsigned ph, int nf, CtaCounts &out) {
+    constexpr int W = 16 / (int)sizeof(CB);
+    unsigned *const pw = st.pw, *const tk = st.tk;
+    int *la = st.la, *lb = st.lb;
+    uint16_t *const won = st.won, *const y = st.y;
+    CB *const ks = st.ks;
+    const int tid = threadIdx.x, nthr = blockDim.x;
+    const int lane = tid & 31, warp = tid >> 5, nwarps = nthr >> 5;
+    int cur = 0;
+    unsigned long long my_cells = 0, my_bytes = 0;  // lane 0's
+    while (nf > T) {
+        if (out.phases >= cap) {
+            out.failed = true;
+            break;
+        }
+        ++out.phases;
+        if (ph == 0xFFFFu) {  // tags are 16 bits: earlier phases' become 1
+#pragma unroll 1
+            for (int a = tid; a < nA; a += nthr)
+                if (pw[a]) pw[a] = 0x10000u | (pw[a] & 0xFFFFu);
+            ph = 1;
+            __syncthreads();
+        }
+        ++ph;
+        const int pp = (int)(out.phases & 1), nxt = cur ^ 1;
+#pragma unroll 1
+        for (int it = warp; it < nf; it += nwarps) {
+            int b = la[it] & kCtaRowMask, start = la[it] >> kCtaRowBits;
+#pragma unroll 1
+            for (;;) {  // one chain: row b from column start, then any row it displaces
+                const CB *row = cb + (size_t)b * ldq;
+                const uint32_t t = cta_target<CB>(y[b]);
+                const int first = start;
+                int found = -1;
+                unsigned old = 0, bytes = 0;
+                uint4 cv[UNROLL];
+#pragma unroll 1
+                for (int c0 = start & ~(W - 1); c0 < ldq && found < 0; c0 += 32 * W * UNROLL) {
+                    cta_load<UNROLL, CB, true>(row, c0, ldq, lane, cv, bytes);
+                    int a;
+#pragma unroll 1
+                    while ((a = cta_test<UNROLL, CB, F7>(cv, ks, tk, c0, start, ldq, t, lane)) >= 0) {
+                        if (lane == 0) old = atomicMax(pw + a, (ph << 16) | (0xFFFFu - (unsigned)b));
+                        old = __shfl_sync(0xFFFFFFFFu, old, 0);
+                        if (old >> 16 != ph || 0xFFFF - (int)(old & 0xFFFFu) > b) {
+                            found = a;
+                            break;
+                        }
+                        start = a + 1;  // a lower row holds it
+                    }
+                }
+                if (lane == 0) {
+                    my_cells += found >= 0 ? (unsigned)(found - first + 1) : (first < nA ? (unsigned)(nA - first) : 0u);
+                    my_bytes += bytes;
+                }
+                const int other = 0xFFFF - (int)(old & 0xFFFFu);
+                if (found >= 0 && old >> 16 == ph) {  // a higher row is displaced: its columns before found are settled
+                    b = other;
+                    start = found + 1;
+                    continue;
+                }
+                if (lane == 0) {
+                    if (found >= 0) {  // found enters M' now; its partner in M, if any, leaves M
+                        won[atomicAdd(&s.nwon[pp], 1)] = (uint16_t)found;
+                        if (old >> 16) lb[atomicAdd(&s.nfl[nxt], 1)] = other | ((found + 1) << kCtaRowBits);
+                    } else {  // y(b) += eps, next phase from column 0
+                        y[b] += 1;
+                        lb[atomicAdd(&s.nfl[nxt], 1)] = b;
+                    }
+                }
+                break;
+            }
+        }
+        ++out.barriers;
+        __syncthreads();
+        const int nwon = s.nwon[pp];
+        nf = s.nfl[nxt];
+#pragma unroll 1
+        for (int i = tid; i < nwon; i += nthr) ks[won[i]] += (CB)1;
+        if (tid == 0) {
+            s.nfl[cur] = 0;      // read at the phase start, filled next phase
+            s.nwon[pp ^ 1] = 0;  // the previous phase's
+        }
+        __syncthreads();
+        int *t = la;
+        la = lb;
+        lb = t;
+        cur = nxt;
+    }
+    out.rounds = out.phases;
+    out.free_at_stop = nf;
+    if (my_cells) atomicAdd(&s.cells, my_cells);
+    if (my_bytes) atomicAdd(&s.bytes, my_bytes);
     __syncthreads();
 }
 

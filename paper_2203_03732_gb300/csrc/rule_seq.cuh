@@ -104,8 +104,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_seq(Params p) {
     };
 
     for (;;) {
-        if ((long long)nf <= p.T) {
-            if (blockIdx.x == 0 && threadIdx.x == 0) ctl->free_at_stop = (int)nf;
+        // (a take-over waits for the first phase: its rows are not in the ring)
+        if ((long long)nf <= p.T || (phase > 0 && (long long)nf <= p.hand)) {
+            if (blockIdx.x == 0 && threadIdx.x == 0) {
+                ctl->free_at_stop = (int)nf;
+                ctl->hand_start = start;  // k_solo takes over the rows from here in the ring
+            }
             break;
         }
         if (phase >= p.phase_cap) {

@@ -69,3 +69,28 @@ def test_crowded_rounds(prot, monkeypatch, eps):
     g = np.random.default_rng(5)
     check(prot, g.random((700, 731)), eps, 1)
     check(prot, np.round(g.random((300, 300)) * 4) / 4, eps, 1)
+
+
+@pytest.mark.parametrize("nB,nA,eps", [(400, 400, 0.1), (1000, 1000, 0.1), (1000, 1010, 0.3), (1024, 1024, 0.05)])
+@pytest.mark.parametrize("squared", [True, False])
+def test_take_over_inside_a_phase(prot, nB, nA, eps, squared):
+    """One phase of many rounds (squared distances: over a hundred): the grid
+    runs its first 16 rounds, one CTA the rest, with the keys, won columns,
+    losers and queued rows of the unfinished phase."""
+    A, B = W.points_uniform(nA, nB, 2, 17 + nB)
+    check(prot, W.pairwise_cost(A, B, squared=squared), eps)
+
+
+@pytest.mark.parametrize("form", ["solo", "hand"])
+@pytest.mark.parametrize("nB,nA,eps", [(33, 33, 5e-5), (300, 300, 0.003), (500, 545, 0.007), (900, 900, 0.01)])
+def test_sequential_greedy_on_one_cta(prot, monkeypatch, form, nB, nA, eps):
+    """Every storage type, and phase tags past 2^16 (84,000 phases)."""
+    import torch
+    monkeypatch.setenv("PR_PHASE_MODE", form)
+    C = W.assignment_euclid_2d(nB, 3 if nB == 33 else 500 + nB, n_a=nA)
+    got = prot.assign(torch.from_numpy(C).cuda(), eps, rule="sequential")
+    ref = oracle.assign(C, eps, mode=oracle.MODE_SEQUENTIAL)
+    for k in ("row_to_col", "col_to_row", "y_row", "y_col"):
+        assert np.array_equal(got[k].cpu().numpy(), ref[k]), k
+    assert got["stats"]["phases"] == ref["stats"]["phases"]
+    assert got["stats"]["free_at_stop"] == ref["stats"]["free_at_stop"]
