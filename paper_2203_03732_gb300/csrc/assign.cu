@@ -69,6 +69,8 @@ constexpr int kMaxCbar8 = 252;
 constexpr int kMaxCbar7 = 125;
 constexpr int kListSm = 1024;             // proposal-list entries kept in shared memory
 constexpr int kKeepMax = 16;              // rows a CTA may keep for its next phase
+constexpr int kFastRows = 4;              // rows of a CTA in a fast round (fast_scan)
+constexpr int kFastUnroll = 5;            // 16-byte loads in flight per lane there: 10 KB over 4 warps
 constexpr int kBatch = 256;               // items turned into scan jobs at a time
 constexpr int kMaxGrid = 1023;            // barrier payload field width
 constexpr unsigned kMidRounds = 16;       // rounds of a phase before k_solo may take over inside it
@@ -280,6 +282,8 @@ struct Smem {
     int job_best[kBatch];
     int2 don[kBatch];         // pool entries given to the pool in this batch
     int best[kWarps];
+    int fbest[kFastRows];     // fast rounds: each row's lowest candidate
+    int4 frow[kFastRows];     // ... (row, scan start, target, 1 if it scanned)
     int nfl[2], nql[2];
     int njob, ndon, don_base;
     int had_prop, nonfirst, nf_delta, donated;
@@ -457,6 +461,55 @@ __device__ __forceinline__ bool grid_sync_pool(Ctl *ctl, Smem &s, unsigned &gen,
     __syncthreads();
     gen += 1;
     return s.err == 0;
+}
+
+// grid_sync_pool for a fast round, run by warp 0 while the other warps wait at
+// the CTA barrier that the caller passes next: the warp's own lanes made the
+// round's proposals and donations, so the arrival needs no CTA barrier before
+// it (__syncwarp orders their writes before lane 0's release).
+__device__ __forceinline__ void warp_sync_pool(Ctl *ctl, Smem &s, unsigned h, unsigned G, long long limit,
+                                               int2 *pool_next, long long pool_base) {
+    const int lane = threadIdx.x & 31;
+    unsigned long long *slot = ctl->bar_slot[h & 3];
+    __syncwarp();
+    unsigned long long v = 0;
+    if (lane == 0) {
+        if (blockIdx.x == 0) {
+            ctl->bar_slot[(h + 2) & 3][0] = 0;
+            ctl->bar_slot[(h + 2) & 3][1] = 0;
+        }
+        const unsigned long long mine = 1ull | ((unsigned long long)s.had_prop << 10) |
+                                        ((unsigned long long)s.nonfirst << 20) |
+                                        ((unsigned long long)s.nf_delta << 40);
+        unsigned long long old;
+        asm volatile("atom.acq_rel.gpu.global.add.u64 %0, [%1], %2;" : "=l"(old) : "l"(slot), "l"(mine) : "memory");
+        v = old + mine;
+        pool_base += (long long)((old >> 40) & 0xFFFFFFull);
+    }
+    pool_base = __shfl_sync(0xFFFFFFFFu, pool_base, 0);
+    for (int i = lane; i < s.ndon; i += 32) pool_put(pool_next, pool_base + i, s.don[i]);
+    if (lane != 0) return;
+    bool ok = true;
+    if ((v & 1023ull) != (unsigned long long)G) {
+        const long long t0 = clock64();
+        for (;;) {
+            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(slot) : "memory");
+            if ((v & 1023ull) == (unsigned long long)G) break;
+            if (ld_relaxed_s32(&ctl->head.abort)) {
+                ok = false;
+                break;
+            }
+            if (clock64() - t0 > limit) {
+                record_error(&ctl->head, PR_ERR_TIMEOUT);
+                ok = false;
+                break;
+            }
+        }
+    }
+    const unsigned long long P = (v >> 10) & 1023ull, L = (v >> 20) & 1023ull;
+    s.pub = ((P ? 1ull : 0ull) << 31) | ((L ? 1ull : 0ull) << 30) | ((v >> 40) & 0xFFFFFFull);
+    s.pub2 = ok ? ((v >> 40) & 0xFFFFFFull) : 0;
+    s.err = ok ? 0 : 1;
 }
 
 // Cluster form of grid_sync, for a launch that is one thread-block cluster.
@@ -850,6 +903,101 @@ __device__ __forceinline__ void run_jobs(Smem &s, const Lists &g, const Params &
 }
 
 // ---------------------------------------------------------------------------
+// A fast round: a CTA with at most kFastRows rows (at n = 10,000, eps = 0.01 all
+// but a few phases have under 500 rows for 152 CTAs).  1, 2 or 4 groups of 16, 8
+// or 4 warps take a row each.  Every warp reads its row's entry itself (the same
+// words in every warp of a group) and issues the row's loads before the round's
+// key update, so the chain entry -> row runs beside it and needs no job list;
+// warp 0's lanes then make the proposals and go straight to the barrier.  A
+// round has 3 CTA barriers instead of 10.  Solve, ms (seed 1 of the sweep): n =
+// 10,000, eps = 0.01 4.18 -> 3.56, eps = 0.005 14.2 -> 12.1; n = 6000, eps = 0.01
+// 3.75 -> 2.79 (with every row to the pool, which it kept from its CTA's next
+// phase before).  Rounds with more rows per CTA pay 0.16 us for the longer
+// code (n = 10,000, eps = 0.1, 147 rounds: 863 -> 887 us).
+// ---------------------------------------------------------------------------
+template <class CB>
+struct FastRow {
+    int b, start, tgt, c0;  // c0: this lane's first column
+    bool act;
+    uint4 v[kFastUnroll];
+};
+
+template <class CB>
+__device__ __forceinline__ void fast_load(const Params &p, FastRow<CB> &f, int c0, int step) {
+    const CB *row = static_cast<const CB *>(p.cb) + (size_t)f.b * p.ldq;
+#pragma unroll
+    for (int u = 0; u < kFastUnroll; ++u) {
+        const int idx = c0 + u * step;
+        if (idx < p.ldq) f.v[u] = ld_nc_na_v4(row + idx);
+    }
+}
+
+// The test of warp_scan_chunk on the group's vectors; the group's lowest
+// candidate goes to s.fbest.
+template <class CB, bool F7>
+__device__ __forceinline__ void fast_scan(Smem &s, const Params &p, const CB *ks, const unsigned *tk, bool check_taken,
+                                          FastRow<CB> &f, int grp, int step, unsigned long long &bytes) {
+    constexpr int W = kPerLoad<CB>;
+    constexpr unsigned kAll = W == 16 ? 0xFFFFu : 0xFFu;
+    const int lane = threadIdx.x & 31;
+    const uint32_t tgt = (uint32_t)f.tgt;
+    const uint32_t t2 = W == 8 ? (tgt | (tgt << 16)) : tgt * 0x01010101u;
+    for (int c = f.c0;;) {
+#pragma unroll
+        for (int u = 0; u < kFastUnroll; ++u) {
+            const int idx = c + u * step;
+            if (__shfl_sync(0xFFFFFFFFu, idx, 0) >= p.ldq) return;  // the warp's lowest column is past the row
+            unsigned m = 0;
+            if (idx < p.ldq) {
+                bytes += 16;
+                const uint4 kv = *reinterpret_cast<const uint4 *>(ks + idx);
+                m = W == 8 ? eq_mask(add_keys(f.v[u], kv), t2) : eq_mask8<F7>(f.v[u], kv, t2);
+                if (m) {
+                    const int lo = f.start - idx;
+                    if (lo > 0) m &= lo >= W ? 0u : (kAll << lo) & kAll;
+                    if (check_taken) m &= ~(tk[idx >> 5] >> (idx & 31)) & kAll;
+                }
+            }
+            const unsigned any = __ballot_sync(0xFFFFFFFFu, m != 0);
+            if (any) {
+                if (lane == __ffs(any) - 1) atomicMin(&s.fbest[grp], idx + __ffs(m) - 1);
+                return;
+            }
+        }
+        c += kFastUnroll * step;
+        volatile int *vb = &s.fbest[grp];
+        if (__shfl_sync(0xFFFFFFFFu, max(c - *vb, c - p.ldq + 1), 0) > 0) return;
+        fast_load<CB>(p, f, c, step);
+    }
+}
+
+// One row's proposal (a >= 0) or relabel by one thread, as run_jobs does it.
+__device__ __forceinline__ void fast_propose(Smem &s, const Lists &g, const Params &p, unsigned *won_now, unsigned R,
+                                             unsigned Rps, int nxt, int qcur, int4 r, int a, unsigned long long &cells) {
+    const int b = r.x, st = r.y, tgt = r.z;
+    cells += a != 0x7FFFFFFF ? (unsigned)(a - st + 1) : (st < p.nA ? (unsigned)(p.nA - st) : 0u);
+    if (a == 0x7FFFFFFF) {
+        atomicAdd(p.y_b + b, 1);  // step (III b): free w.r.t. M' -> relabel
+        push_next(s, nxt, 0, b, tgt + 2);
+        return;
+    }
+    const unsigned long long old = atomicMax(p.prop + a, word_of(R, b));
+    const unsigned t = tag_of(old);
+    if (t < Rps) {
+        atomicOr(won_now + (a >> 5), 1u << (a & 31));
+        atomicAdd(reinterpret_cast<unsigned *>(p.ka + (a & ~1)), (a & 1) ? 0x10000u : 1u);
+        const int partner = row_of(old);
+        if (partner >= 0) push_next(s, nxt, 0, partner, -2 - a);
+    } else if (t == R) {
+        s.nonfirst = 1;
+    } else {
+        record_error(&p.ctl->head, PR_ERR_INTERNAL);
+    }
+    ql_push(s, g, qcur, b, a, tgt + 1, 0);
+    s.had_prop = 1;
+}
+
+// ---------------------------------------------------------------------------
 // k_phases: every phase of Sec. 2.2 in one cooperative launch.
 //
 // Phase 0 deals rows b = cta + k*G.  Afterwards each CTA keeps up to `keep`
@@ -890,10 +1038,10 @@ k_phases(Params p, int warps_per_row, int rows_per_group) {
     Ctl *ctl = p.ctl;
     const unsigned G = gridDim.x;
     const int cta = blockIdx.x;
-    // With at most two rows per register group (long rows) every free row
-    // goes to the pool, which deals them out evenly (measured at n = 10,000:
-    // 1-3 % faster than keeping one); shorter rows keep up to a group's worth.
-    const int keep = rows_per_group > 2 && p.hand == 0 && p.mid == 0 ? min(rows_per_group - 1, kKeepMax) : 0;
+    // Every free row goes to the pool, which deals them out evenly, and the
+    // rounds of few rows are fast ones; the forms without them keep up to a
+    // register group's worth of rows when rows are short.
+    const int keep = (OFS || CL || p.nB > kBatch * (int)G) && rows_per_group > 2 ? min(rows_per_group - 1, kKeepMax) : 0;
     // Every next-phase row goes to the pool and no CTA takes more than kBatch
     // rows in a round (so its donations of a round fit s.don): the barrier
     // places the donations (grid_sync_pool).
@@ -940,6 +1088,8 @@ k_phases(Params p, int warps_per_row, int rows_per_group) {
     // started and zeroed them.
     if (CL) cluster_barrier_hw();
 
+    const bool fast_ok = !OFS && place_at_barrier && !p.profile;
+    unsigned long long fast_bytes = 0, fast_rows = 0;  // this thread's, added up at exit
     unsigned gen = 0;
     unsigned R = 0;  // global round counter (round tags)
     long long phase = 0, rounds = 0;
@@ -972,13 +1122,58 @@ k_phases(Params p, int warps_per_row, int rows_per_group) {
             }
             // items of this round: kept rows + pool share, or last round's proposals
             const int nitems = first_round ? kept + from_pool : s.nql[qcur ^ 1];
+            // a fast round: the row of this warp's group, its loads in flight
+            const bool fast = fast_ok && nitems <= kFastRows;
+            const int f_wpg = nitems <= 1 ? kWarps : nitems <= 2 ? kWarps / 2 : kWarps / 4;  // warps per row
+            const int f_grp = f_wpg == kWarps ? 0 : (int)(threadIdx.x >> 5) / f_wpg;
+            const int f_step = f_wpg * 32 * kPerLoad<CB>;
+            FastRow<CB> f;
+            if (fast) {
+                if (threadIdx.x < kFastRows) s.fbest[threadIdx.x] = 0x7FFFFFFF;
+                f.act = f_grp < nitems;
+                int y = 1;
+                f.b = f.start = 0;
+                if (f.act) {
+                    if (!first_round) {
+                        const int4 q = s.ql[qcur ^ 1][f_grp];
+                        f.b = q.x;
+                        f.start = q.y + 1;
+                        y = q.z;
+                        f.act = row_of(ld_relaxed_u64(p.prop + q.y)) != q.x;  // else it won: matched, leaves B'
+                    } else if (phase == 0) {
+                        f.b = cta + f_grp * (int)G;
+                    } else {
+                        unsigned long long raw = pool_raw(pool_now, cta + (long long)f_grp * G);
+                        const long long t0 = clock64();
+                        while ((unsigned)(raw >> 32) == 0u) {  // as pool_take
+                            if (clock64() - t0 > p.spin_limit) {
+                                record_error(&ctl->head, PR_ERR_TIMEOUT);
+                                break;
+                            }
+                            raw = pool_raw(pool_now, cta + (long long)f_grp * G);
+                        }
+                        f.act = (unsigned)(raw >> 32) != 0u;  // else the kernel stops at the next barrier
+                        f.b = f.act ? (int)(unsigned)raw : 0;
+                        y = f.act ? (int)(raw >> 32) : 1;
+                    }
+                }
+                if (y < 0) f.start = -1 - y;
+                f.act = __all_sync(0xFFFFFFFFu, f.act);
+                f.c0 = (f.start & ~(kPerLoad<CB> - 1)) +
+                       ((int)(threadIdx.x >> 5) - f_grp * f_wpg) * 32 * kPerLoad<CB> + (int)(threadIdx.x & 31) * kPerLoad<CB>;
+                f.tgt = y - 1;
+                if (f.act) {
+                    fast_load<CB>(p, f, f.c0, f_step);
+                    if (y < 0) f.tgt = ld_relaxed_s32(p.y_b + f.b) - 1;
+                }
+            }
             // Issue this thread's first item load and its bitmap-word load
             // before using either, so the two global reads overlap.
             unsigned long long pre_pool = 0;
             unsigned long long pre_word = 0;
             int4 pre_q = make_int4(0, 0, 0, 0);
             const int it0 = threadIdx.x;
-            if (it0 < nitems && it0 < kBatch) {
+            if (!fast && it0 < nitems && it0 < kBatch) {
                 if (first_round) {
                     if (phase > 0 && it0 >= kept)
                         pre_pool = pool_raw(pool_now, cta + (long long)(it0 - kept) * G);
@@ -1012,6 +1207,30 @@ k_phases(Params p, int warps_per_row, int rows_per_group) {
                     wold[i] = 0;
             }
             __syncthreads();
+            if (fast) {
+                if (f.act) {
+                    fast_scan<CB, F7>(s, p, ks, tk, !first_round, f, f_grp, f_step, fast_bytes);
+                }
+                if ((int)threadIdx.x == f_grp * f_wpg * 32) {  // the group's first thread
+                    s.frow[f_grp] = make_int4(f.b, f.start, f.tgt, f.act ? 1 : 0);
+                    // the slot is free again: every warp of the group has its entry
+                    if (first_round && phase > 0 && f.act && f_grp < nitems)
+                        s.frow[f_grp].w = 2;
+                }
+                __syncthreads();
+                if (threadIdx.x < 32) {
+                    if ((int)threadIdx.x < nitems && s.frow[threadIdx.x].w != 0) {
+                        const int4 r = s.frow[threadIdx.x];
+                        if (r.w == 2) pool_put(pool_now, cta + (long long)threadIdx.x * G, make_int2(0, 0));
+                        fast_propose(s, g, p, won_now, R, Rps, cur ^ 1, qcur, r, s.fbest[threadIdx.x], cells);
+                        ++fast_rows;
+                    }
+                    warp_sync_pool(ctl, s, gen + 1, G, p.spin_limit, pool_next, pool_next_size);
+                }
+                ++gen;
+                __syncthreads();
+                if (s.err) goto done;
+            } else {
             const unsigned long long t_r1 = p.profile ? ptimer() : 0;
             unsigned long long t_mark = t_r1;
             // PR_RULE_OFFSET turns a row into up to two jobs: half as many per batch
@@ -1121,6 +1340,7 @@ k_phases(Params p, int warps_per_row, int rows_per_group) {
                     ctl->prof_rounds += 1;
                 }
             }
+            }
             const unsigned long long pub = s.pub;
             if ((pub >> 31) & 1ull) ++rounds;
             nf_next += (long long)(pub & 0x3FFFFFFFull);
@@ -1161,6 +1381,8 @@ k_phases(Params p, int warps_per_row, int rows_per_group) {
     }
 done:
     if (cells) atomicAdd(&s.cells, cells);
+    if (fast_bytes) atomicAdd(&s.bytes, fast_bytes);
+    if (fast_rows) atomicAdd(&s.rows, fast_rows);
     __syncthreads();
     if (threadIdx.x == 0) {
         if (s.bytes) atomicAdd(&ctl->bytes, s.bytes);
