@@ -290,10 +290,18 @@ struct BatchCost {
     }
 };
 
+// CTAs per SM the registers are held to: 128 registers a thread at 128 and 256
+// threads, so that 4 and 2 CTAs fit (the compiler takes 172 otherwise, and one
+// CTA of 256 threads sat alone on an SM: 512 problems of up to 2048 rows 2.69
+// -> 2.00 ms).  85 and 64 registers spill: that batch 1.90 and 1.86 ms, but 300
+// problems of up to 700 rows 0.73 -> 0.85 and 0.91 ms.
+template <int THREADS>
+constexpr int kSolveCtas = THREADS == 128 ? 4 : THREADS == 256 ? 2 : 1;
+
 // F7: floor(1/eps) <= 125, so every sum of a real column's cbar and key
 // stays below 256 and the byte pre-test is one plain add (may_match<true>).
 template <int THREADS, int UNROLL, class CB, bool F7>
-__global__ void __launch_bounds__(THREADS, 1) k_bsolve(BParams p) {
+__global__ void __launch_bounds__(THREADS, kSolveCtas<THREADS>) k_bsolve(BParams p) {
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ CtaShared s;
     __shared__ int cur_problem;
@@ -419,12 +427,16 @@ pr_status run_batched(const Source &src, int32_t P, const int32_t *n_host, doubl
     if (!ws || ((uintptr_t)ws & 255) || ws_bytes < L.total)
         return fail(PR_ERR_WORKSPACE, "batched: workspace NULL, not 256-byte aligned or < %zu bytes", L.total);
     // Threads per CTA by the largest problem: short rows and few of them want
-    // cheap CTA barriers and many problems per SM, larger problems more warps
-    // (eps = 0.01, ms at 128 / 256 / 512 threads: 512 problems up to 300 rows
-    // 0.95 / 1.40 / 1.44, 300 up to 700: 1.04 / 1.07 / 1.11, 100 up to 1024:
-    // 0.94 / 0.65 / 0.60, 512 up to 2048: 2.69 / 3.04 / 2.67).  The order of
-    // the cost sum stays that of kCostSums partial sums.
-    int threads = pl.n_max <= 400 ? 128 : pl.n_max <= 700 ? 256 : 512, per_sm_want = 0;
+    // cheap CTA barriers and many problems per SM, larger problems more warps,
+    // unless there are more problems than SMs and rounds are small (eps = 0.01,
+    // ms at 128 / 256 / 512 threads: 512 problems up to 300 rows 0.95 / 1.15 /
+    // 1.44; 300 up to 700: 1.03 / 0.73 / 1.09; 100 up to 1024: 0.93 / 0.64 / 0.59;
+    // 512 up to 2048: 2.37 / 2.00 / 2.32; at eps = 0.1, 300 up to 1500: 1.27 /
+    // 0.87 / 0.66).  The order of the cost sum stays that of kCostSums partial
+    // sums.
+    const DeviceInfo &di = device_info();
+    const bool many = P > di.sms && floor(1.0 / eps) > 20.0;
+    int threads = pl.n_max <= 400 ? 128 : pl.n_max <= 700 || many ? 256 : 512, per_sm_want = 0;
     int cost_sums = kCostSums;
     if (tune) {
         if (tune->threads) cost_sums = threads = tune->threads;
@@ -442,8 +454,6 @@ pr_status run_batched(const Source &src, int32_t P, const int32_t *n_host, doubl
     unsigned *d_max = (unsigned *)(w + L.maxbits);
     void *d_cb = w + L.cb;
     const bool cb8 = floor(1.0 / eps) <= (double)kMaxCbarByte;
-    const DeviceInfo &di = device_info();
-
     k_binit<<<(P + 255) / 256, 256, 0, st>>>(ctl, d_max, P);
     PR_CUDA(cudaGetLastError());
     // problem table: copied from pageable host memory (waits for earlier work
