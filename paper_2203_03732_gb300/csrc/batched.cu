@@ -18,6 +18,7 @@
 
 #include <algorithm>
 #include <numeric>
+#include <type_traits>
 #include <vector>
 
 #include "prot_internal.cuh"
@@ -139,7 +140,7 @@ __global__ void __launch_bounds__(256, 4) k_bquant_matrix(const T *__restrict__ 
 // kPtRows pairs and the rounded costs are stored 4 (16-bit storage: 8) bytes at
 // a time; the squared sum keeps the operation order of dist_f32.  DIM = 0: any
 // dimension, one pair at a time.  64 clouds of 4096 3-D points (1.07 G pairs):
-// largest distance 0.96 -> 0.35 ms, rounding 2.20 -> 0.82 ms (three loads and about
+// largest distance 0.96 -> 0.35 ms, rounding 2.20 -> 0.68 ms (three loads and about
 // 60 instructions a pair before).
 // ---------------------------------------------------------------------------
 constexpr int kPtRows = 8;
@@ -224,14 +225,15 @@ __global__ void __launch_bounds__(256, 4) k_bpoints_max(const float *__restrict_
     });
 }
 
-template <int DIM, class CB>
-__global__ void __launch_bounds__(256, 3) k_bpoints_quant(const float *__restrict__ XA, const float *__restrict__ XB, int dim,
-                                int squared, const BDesc *__restrict__ d, int P, int total_rows,
+constexpr int kPointCtas = 3;  // CTAs of k_bpoints_quant per SM, by its registers
+template <int DIM, bool SQ, class CB>
+__global__ void __launch_bounds__(256, kPointCtas) k_bpoints_quant(const float *__restrict__ XA, const float *__restrict__ XB, int dim,
+                                const BDesc *__restrict__ d, int P, int total_rows,
                                 const unsigned *__restrict__ maxbits, EpsSplit e, CB *__restrict__ cb) {
     const int lane = threadIdx.x & 31;
     point_tiles(d, P, total_rows, [&](int i, int r, int rows) {
         const BDesc D = d[i];
-        const PointsScale ps = points_scale(maxbits[i], squared, e);
+        const PointsScale ps = points_scale(maxbits[i], SQ, e);
         CB *out = cb + D.cb_off + (long long)(r - D.v_off) * D.ldq;
         if constexpr (DIM == 0) {
             for (int q = 0; q < rows; ++q)
@@ -239,7 +241,7 @@ __global__ void __launch_bounds__(256, 3) k_bpoints_quant(const float *__restric
                     uint32_t h = kPadOf<CB>;
                     if (a < D.n) {
                         const float dd =
-                            dist_f32(XB + (long long)(r + q) * dim, XA + (long long)(D.v_off + a) * dim, dim, squared);
+                            dist_f32(XB + (long long)(r + q) * dim, XA + (long long)(D.v_off + a) * dim, dim, SQ);
                         const float c = ps.M > 0.0f ? __fdiv_rn(dd, ps.M) : 0.0f;
                         h = quantise_fbits(__float_as_uint(c), e);
                     }
@@ -257,10 +259,12 @@ __global__ void __launch_bounds__(256, 3) k_bpoints_quant(const float *__restric
                     float sq[4];
                     uint32_t h[4];
                     sq_group4<DIM>(xb[q], xa, sq);
-                    quantise_points<4>(sq, squared, ps, e, h, [](float, uint32_t k) { return k; });
+                    quantise_points<4>(sq, SQ, ps, e, h, [](float, uint32_t k) { return k; });
+                    if (a + 4 > D.n) {
 #pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        if (a + j >= D.n) h[j] = kPadOf<CB>;
+                        for (int j = 0; j < 4; ++j)
+                            if (a + j >= D.n) h[j] = kPadOf<CB>;
+                    }
                     CB *o = out + (long long)q * D.ldq + a;
                     if (sizeof(CB) == 1)
                         *reinterpret_cast<uint32_t *>(o) = pack_bytes(h[0], h[1], h[2], h[3]);
@@ -471,26 +475,33 @@ pr_status run_batched(const Source &src, int32_t P, const int32_t *n_host, doubl
         const int D = src.dim == 2 ? 2 : src.dim == 3 ? 3 : 0;
         const void *kmax = D == 2 ? (const void *)k_bpoints_max<2> : D == 3 ? (const void *)k_bpoints_max<3>
                                                                               : (const void *)k_bpoints_max<0>;
-        const void *kq = cb8 ? (D == 2 ? (const void *)k_bpoints_quant<2, uint8_t>
-                                : D == 3 ? (const void *)k_bpoints_quant<3, uint8_t>
-                                         : (const void *)k_bpoints_quant<0, uint8_t>)
-                             : (D == 2 ? (const void *)k_bpoints_quant<2, uint16_t>
-                                : D == 3 ? (const void *)k_bpoints_quant<3, uint16_t>
-                                         : (const void *)k_bpoints_quant<0, uint16_t>);
-        int dim_ = src.dim, sq_ = src.squared, P_ = P, rows_ = pl.v_total;
+        const auto quant = [&](auto d_, auto sq_) -> const void * {
+            constexpr int kD = decltype(d_)::value;
+            constexpr bool kSq = decltype(sq_)::value;
+            return cb8 ? (const void *)k_bpoints_quant<kD, kSq, uint8_t> : (const void *)k_bpoints_quant<kD, kSq, uint16_t>;
+        };
+        const auto quant_d = [&](auto d_) {
+            return src.squared ? quant(d_, std::true_type{}) : quant(d_, std::false_type{});
+        };
+        const void *kq = D == 2   ? quant_d(std::integral_constant<int, 2>{})
+                         : D == 3 ? quant_d(std::integral_constant<int, 3>{})
+                                  : quant_d(std::integral_constant<int, 0>{});
+        int dim_ = src.dim, P_ = P, rows_ = pl.v_total;
         const float *xa_ = src.XA, *xb_ = src.XB;
         const BDesc *dd_ = d_desc;
         unsigned *mx_ = d_max;
         // a warp per kPtRows rows
-        const int pgrid = std::max(1, std::min(di.sms * 4, (pl.v_total + 8 * kPtRows - 1) / (8 * kPtRows)));
+        // (no more CTAs than are resident: a second wave of the rounding took 0.81
+        // against 0.68 ms at 64 clouds of 4096 points)
+        const int tiles = std::max(1, (pl.v_total + 8 * kPtRows - 1) / (8 * kPtRows));
         void *amax[] = {(void *)&xa_, (void *)&xb_, (void *)&dim_, (void *)&dd_, (void *)&P_, (void *)&rows_,
                         (void *)&mx_};
-        PR_CUDA(cudaLaunchKernel(kmax, dim3(pgrid), dim3(256), amax, 0, st));
+        PR_CUDA(cudaLaunchKernel(kmax, dim3(std::min(di.sms * 4, tiles)), dim3(256), amax, 0, st));
         const unsigned *cmx_ = d_max;
         void *cbp_ = d_cb;
-        void *aq[] = {(void *)&xa_, (void *)&xb_, (void *)&dim_, (void *)&sq_, (void *)&dd_, (void *)&P_,
+        void *aq[] = {(void *)&xa_, (void *)&xb_, (void *)&dim_, (void *)&dd_, (void *)&P_,
                       (void *)&rows_, (void *)&cmx_, (void *)&e, (void *)&cbp_};
-        PR_CUDA(cudaLaunchKernel(kq, dim3(pgrid), dim3(256), aq, 0, st));
+        PR_CUDA(cudaLaunchKernel(kq, dim3(std::min(di.sms * kPointCtas, tiles)), dim3(256), aq, 0, st));
     } else if (src.dt == PR_F64) {
         if (cb8)
             k_bquant_matrix<double, uint8_t><<<qgrid, 256, 0, st>>>((const double *)src.C, d_desc, P, pl.v_total, e,
