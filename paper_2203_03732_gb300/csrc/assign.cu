@@ -103,6 +103,7 @@ struct Ctl {
     unsigned long long prof_rounds;
     unsigned long long seq_tail;  // PR_RULE_SEQUENTIAL: rows queued so far (rule_seq.cuh)
     unsigned long long hand_start;  // and, at a take-over, the first of them that is still to run
+    unsigned cost_done;  // CTAs of k_cost that have finished
     int mid_rows;      // take-over inside a phase: rows that lost the last round (in p.lists)
     unsigned mid_rps;  // ... and the phase's first round
 };
@@ -113,7 +114,7 @@ constexpr int kProfSegs = 7;
 __device__ __forceinline__ unsigned long long ptimer() { return (unsigned long long)clock64(); }
 
 struct Layout {
-    size_t ctl, cb, ka, prop, won, pool, lists, ii, total;
+    size_t ctl, cb, ka, prop, won, pool, part, lists, ii, total;
     int ldq, won_words;
     size_t list_stride;  // ints per CTA in the list region
 };
@@ -132,6 +133,7 @@ Layout make_layout(int nB, int nA, int grid) {
     L.won_words = (nA + 31) / 32;
     L.won = c.take<unsigned>(3 * (size_t)L.won_words);
     L.pool = c.take<int2>(2 * (size_t)nB);
+    L.part = c.take<double>(1024);
     L.list_stride = 8 * (size_t)nB;
     L.lists = c.take<int>((size_t)grid * L.list_stride);
     // PR_RULE_ISRAELI_ITAI's state (rule_ii.cuh): 28 bytes per column, 36 per row
@@ -161,6 +163,7 @@ struct Params {
                        // 2 Israeli-Itai, 3 the sequential greedy by displacement chains
     void *ii = nullptr;  // PR_RULE_ISRAELI_ITAI's state region
     int near = 0;  // floor(1/eps) <= kNearMaxK: later rounds' scans are short (near_scans)
+    double *part = nullptr;  // k_cost's partial sums
     int mid = 0;   // k_phases stops inside a phase of kMidRounds rounds, and k_solo goes on
     int hand = 0;  // k_phases stops at this many free rows, all in the pool, and k_solo goes on (0: never)
 };
@@ -1425,32 +1428,67 @@ __global__ void k_decode(Params p, int *match_b, int *match_a, int *y_col) {
 }
 
 // ---------------------------------------------------------------------------
-// k_finish (one CTA): completion (k-th free row with k-th free column) and the
-// FP64 matching cost with a fixed-order tree reduction.
+// k_finish (one CTA): completion (k-th free row with k-th free column) and,
+// with COST, the FP64 matching cost: kFinThreads strided partial sums and a
+// halving tree.  Bound by its chain of scans, so a thread takes 4 rows a step.
+// k_cost: the same sum spread over kCostCtas CTAs, 32 partial sums to each, the
+// tree run by the CTA that finishes last (the same order, the same bits).  For
+// costs from points, whose distances keep one SM's few FP64 units busy: n =
+// 10,000 78 us in one CTA with the completion, now 34 us in both; a matrix's
+// costs are a gather, for which a second launch gains nothing (30.6 -> 20.5 us
+// in one CTA).
 // ---------------------------------------------------------------------------
 constexpr int kFinThreads = 1024;
+constexpr int kCostCtas = kFinThreads / 32;
 
-__device__ __forceinline__ int block_exclusive_scan(int flag, int *warp_tot, int *total) {
+// Exclusive prefix sum of c over the CTA; *total receives the sum.
+__device__ __forceinline__ int block_exclusive_sum(int c, int *warp_tot, int *total) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const unsigned bal = __ballot_sync(0xFFFFFFFFu, flag);
-    const int within = __popc(bal & ((1u << lane) - 1));
-    if (lane == 0) warp_tot[warp] = __popc(bal);
+    int x = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) warp_tot[warp] = x;
     __syncthreads();
     if (warp == 0) {
         const int v = lane < (kFinThreads / 32) ? warp_tot[lane] : 0;
-        int x = v;
+        int z = v;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-            if (lane >= o) x += y;
+            const int y = __shfl_up_sync(0xFFFFFFFFu, z, o);
+            if (lane >= o) z += y;
         }
-        if (lane < (kFinThreads / 32)) warp_tot[lane] = x - v;
-        if (lane == 31) *total = x;
+        if (lane < (kFinThreads / 32)) warp_tot[lane] = z - v;
+        if (lane == 31) *total = z;
     }
     __syncthreads();
-    const int r = warp_tot[warp] + within;
+    const int r = warp_tot[warp] + x - c;
     __syncthreads();
     return r;
+}
+
+// The first `cap` indices i < n with match[i] < 0, ascending; returns how many.
+__device__ __forceinline__ int list_free(const int *match, int n, int cap, int *out, int *warp_tot, int *total) {
+    int found = 0;
+    for (int base = 0; base < n && found < cap; base += 4 * kFinThreads) {
+        const int i0 = base + 4 * threadIdx.x;
+        unsigned f = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (i0 + k < n && match[i0 + k] < 0) f |= 1u << k;
+        int pos = found + block_exclusive_sum(__popc(f), warp_tot, total);
+        found += *total;
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if ((f >> k) & 1u) {
+                if (pos < cap) out[pos] = i0 + k;
+                ++pos;
+            }
+        __syncthreads();  // *total has been read
+    }
+    return min(found, cap);
 }
 
 // The matched costs k_finish adds up: from the input matrix, or the FP64
@@ -1469,37 +1507,24 @@ struct PointsCost {
     }
 };
 
-template <class Src>
+template <bool COST, class Src>
 __global__ void __launch_bounds__(kFinThreads)
 k_finish(Params p, Src src, int *match_b, int *match_a, int *free_b, int *free_a, double *cost) {
     __shared__ int warp_tot[32];
     __shared__ int total;
-    __shared__ double part[kFinThreads];
+    __shared__ double part[COST ? kFinThreads : 1];
     if (ld_relaxed_s32(&p.ctl->head.err) != 0) return;
-    int nfb = 0;
-    for (int base = 0; base < p.nB; base += kFinThreads) {
-        const int b = base + threadIdx.x;
-        const int f = (b < p.nB && match_b[b] < 0) ? 1 : 0;
-        const int pos = block_exclusive_scan(f, warp_tot, &total);
-        if (f) free_b[nfb + pos] = b;
-        nfb += total;
-        __syncthreads();
-    }
-    int nfa = 0;
-    for (int base = 0; base < p.nA && nfa < nfb; base += kFinThreads) {
-        const int a = base + threadIdx.x;
-        const int f = (a < p.nA && match_a[a] < 0) ? 1 : 0;
-        const int pos = block_exclusive_scan(f, warp_tot, &total);
-        if (f && nfa + pos < nfb) free_a[nfa + pos] = a;
-        nfa += total;
-        __syncthreads();
-    }
+    const int nfb = list_free(match_b, p.nB, p.nB, free_b, warp_tot, &total);
+    list_free(match_a, p.nA, nfb, free_a, warp_tot, &total);
+    __syncthreads();
     for (int k = threadIdx.x; k < nfb; k += kFinThreads) {
         match_b[free_b[k]] = free_a[k];
         match_a[free_a[k]] = free_b[k];
     }
+    if (!COST) return;
     __syncthreads();
     double acc = 0.0;
+#pragma unroll 4
     for (int b = threadIdx.x; b < p.nB; b += kFinThreads)
         acc = __dadd_rn(acc, src(b, match_b[b]));
     part[threadIdx.x] = acc;
@@ -1509,6 +1534,30 @@ k_finish(Params p, Src src, int *match_b, int *match_a, int *free_b, int *free_a
         __syncthreads();
     }
     if (threadIdx.x == 0) *cost = part[0];
+}
+
+template <class Src>
+__global__ void __launch_bounds__(32) k_cost(Params p, Src src, const int *match_b, double *cost) {
+    __shared__ double part[kFinThreads];
+    if (ld_relaxed_s32(&p.ctl->head.err) != 0) return;
+    const int lane = threadIdx.x, v = blockIdx.x * 32 + lane;
+    double acc = 0.0;
+#pragma unroll 4
+    for (int b = v; b < p.nB; b += kFinThreads) acc = __dadd_rn(acc, src(b, match_b[b]));
+    p.part[v] = acc;
+    __threadfence();
+    unsigned last = 0;
+    if (lane == 0) last = atomicAdd(&p.ctl->cost_done, 1u) == gridDim.x - 1 ? 1u : 0u;
+    if (!__shfl_sync(0xFFFFFFFFu, last, 0)) return;
+    __threadfence();
+    const volatile double *q = p.part;
+    for (int i = lane; i < kFinThreads; i += 32) part[i] = q[i];
+    __syncwarp();
+    for (int w = kFinThreads / 2; w > 0; w >>= 1) {
+        for (int i = lane; i < w; i += 32) part[i] = __dadd_rn(part[i], part[i + w]);
+        __syncwarp();
+    }
+    if (lane == 0) *cost = part[0];
 }
 
 // ---------------------------------------------------------------------------
@@ -2186,17 +2235,19 @@ pr_status launch_solve(Params &p, const CostSource &src, double eps, const Phase
     // completion scratch: the first CTA's list region (free after the loop)
     int *free_b = p.lists;
     int *free_a = p.lists + n_rows;
-    if (solo || take_over) {
-        // done by k_solo
-    } else if (src.points)
-        k_finish<PointsCost><<<1, kFinThreads, 0, st>>>(p, PointsCost{src.XA, src.XB, src.dim, src.squared},
-                                                         row_to_col, col_to_row, free_b, free_a, cost);
-    else if (dt == PR_F64)
-        k_finish<MatrixCost<double>><<<1, kFinThreads, 0, st>>>(p, MatrixCost<double>{(const double *)C, ldc},
-                                                                row_to_col, col_to_row, free_b, free_a, cost);
-    else
-        k_finish<MatrixCost<float>><<<1, kFinThreads, 0, st>>>(p, MatrixCost<float>{(const float *)C, ldc},
-                                                               row_to_col, col_to_row, free_b, free_a, cost);
+    if (!solo && !take_over) {  // else k_solo has done both
+        if (src.points) {
+            const PointsCost pc{src.XA, src.XB, src.dim, src.squared};
+            k_finish<false><<<1, kFinThreads, 0, st>>>(p, pc, row_to_col, col_to_row, free_b, free_a, cost);
+            k_cost<<<kCostCtas, 32, 0, st>>>(p, pc, row_to_col, cost);
+        } else if (dt == PR_F64) {
+            k_finish<true><<<1, kFinThreads, 0, st>>>(p, MatrixCost<double>{(const double *)C, ldc}, row_to_col,
+                                                      col_to_row, free_b, free_a, cost);
+        } else {
+            k_finish<true><<<1, kFinThreads, 0, st>>>(p, MatrixCost<float>{(const float *)C, ldc}, row_to_col,
+                                                      col_to_row, free_b, free_a, cost);
+        }
+    }
     PR_CUDA(cudaGetLastError());
 
     if (stats) {
@@ -2293,6 +2344,7 @@ pr_status assign_common(const CostSource &src, int32_t n_rows, int32_t n_cols, d
     p.won = (unsigned *)(w + L.won);
     p.won_words = L.won_words;
     p.pool = (int2 *)(w + L.pool);
+    p.part = (double *)(w + L.part);
     p.lists = (int *)(w + L.lists);
     p.list_stride = L.list_stride;
     p.nB = n_rows;
@@ -2424,7 +2476,7 @@ constexpr size_t kNoAllocBytes = (size_t)2304 * 1024;
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
 
 struct NoAllocLayout {
-    size_t ctl, cb, ka, prop, won, pool, lists, total;
+    size_t ctl, cb, ka, prop, won, pool, part, lists, total;
     int ldq, won_words;
 };
 
@@ -2441,6 +2493,7 @@ NoAllocLayout make_noalloc_layout(int nB, int nA) {
     L.won_words = (nA + 31) / 32;
     L.won = c.take<unsigned>(3 * (size_t)L.won_words);
     L.pool = c.take<int2>(2 * (size_t)nB);
+    L.part = c.take<double>(1024);
     L.lists = c.take<int>(2 * (size_t)nB);  // completion scratch
     L.total = c.total();
     return L;
@@ -2501,6 +2554,7 @@ extern "C" pr_status pr_assign_noalloc(const void *C, pr_dtype dt, int64_t ldc, 
     p.won = (unsigned *)(w + L.won);
     p.won_words = L.won_words;
     p.pool = (int2 *)(w + L.pool);
+    p.part = (double *)(w + L.part);
     p.lists = (int *)(w + L.lists);
     p.list_stride = 0;  // no overflow region: never addressed for n_rows <= 1024
     p.nB = n_rows;
