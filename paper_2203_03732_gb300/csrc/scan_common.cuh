@@ -261,16 +261,6 @@ __device__ __forceinline__ uint32_t byte_marks(uint32_t c, uint32_t k, uint32_t 
     const uint32_t ovf = (c & k) | ((c | k) & s7);  // bit 7: carry out of bit 7
     return zero & ~ovf;
 }
-__device__ __forceinline__ unsigned byte_bits(uint32_t w) {  // bit i = low bit of byte i
-    return ((w & 0x01010101u) * 0x01020408u) >> 24;
-}
-// Bit j of the result is set iff byte j of c + k equals the target (t4 =
-// target in all four bytes), for the sixteen bytes of one 16-byte load.
-__device__ __forceinline__ unsigned eq_mask8_exact(uint4 c, uint4 k, uint32_t t4) {
-    const uint32_t a = byte_marks(c.x, k.x, t4), b = byte_marks(c.y, k.y, t4);
-    const uint32_t d = byte_marks(c.z, k.z, t4), e = byte_marks(c.w, k.w, t4);
-    return byte_bits(a >> 7) | (byte_bits(b >> 7) << 4) | (byte_bits(d >> 7) << 8) | (byte_bits(e >> 7) << 12);
-}
 // A first test that most loads settle: nonzero iff some byte of the four
 // words may match.  (z - 0x01..) & ~z & 0x80.. is nonzero iff some byte of
 // z is zero (exact as an existence test).  F7 (floor(1/eps) <= 125: cbar <=
@@ -284,20 +274,12 @@ __device__ __forceinline__ uint32_t may_match(uint32_t c, uint32_t k, uint32_t t
     if (F7) return zero_byte((c + k) ^ t4);
     return zero_byte((((c & 0x7F7F7F7Fu) + (k & 0x7F7F7F7Fu)) ^ ((c ^ k) & 0x80808080u)) ^ t4);
 }
-template <bool F7 = false>
-__device__ __forceinline__ unsigned eq_mask8(uint4 c, uint4 k, uint32_t t4) {
-    if ((may_match<F7>(c.x, k.x, t4) | may_match<F7>(c.y, k.y, t4) | may_match<F7>(c.z, k.z, t4) |
-         may_match<F7>(c.w, k.w, t4)) == 0u)
-        return 0u;
-    return eq_mask8_exact(c, k, t4);
-}
-
 // The exact test without a branch, for scans that find a candidate in most
 // vectors: bit j of the result is set iff column j of the vector has cbar + k
 // == target.  Per word 5 operations mark the zero bytes (halves) of z = (c +
 // k) ^ t at their top bit, and one dp4a gathers a word's marks into bits
 // (0x80 per marked byte times a power of two, summed), 27 instructions per
-// 16 bytes against about 70 for the pre-test and eq_mask8_exact together.
+// 16 bytes against about 70 for four multiplications that gather byte by byte.
 // 16-bit values: cbar + k <= 65534 never carries between halves (padding
 // 0x7FFF + 0x8000).  Bytes with F7: real columns' sums stay below 256 and
 // padding bytes sit above them; otherwise byte_marks masks the carries.
@@ -325,6 +307,14 @@ __device__ __forceinline__ unsigned vec_marks(uint4 c, uint4 k, uint32_t t) {
     m = __dp4a(half_marks(c.z + k.z, t), 0x20001000u, m);
     m = __dp4a(half_marks(c.w + k.w, t), 0x80004000u, m);
     return m >> 7;
+}
+// Bytes: the pre-test, then the exact marks for the loads that pass it.
+template <bool F7 = false>
+__device__ __forceinline__ unsigned eq_mask8(uint4 c, uint4 k, uint32_t t4) {
+    if ((may_match<F7>(c.x, k.x, t4) | may_match<F7>(c.y, k.y, t4) | may_match<F7>(c.z, k.z, t4) |
+         may_match<F7>(c.w, k.w, t4)) == 0u)
+        return 0u;
+    return vec_marks<uint8_t, F7>(c, k, t4);
 }
 // A test that never misses a candidate: nonzero if some column of the vector
 // may match (16-bit values and F7: exactly if one does).
