@@ -6,7 +6,9 @@
 //               floor(1/eps) <= 252, else uint16                   (Eq. 1)
 //   k_phases    persistent cooperative kernel: every phase and round
 //   k_decode    matching and y(A) out of the per-column words
-//   k_finish    completion + FP64 cost                             (Sec. 2.1)
+//   k_finish    completion + FP64 cost (points: k_cost)             (Sec. 2.1)
+// Small problems: k_solo (cta_solve.cuh) runs the phases on one CTA, or takes
+// them over from k_phases, and does what follows as well (use_cta).
 //
 // Integer form (units of eps): with k(a) = -y(a) >= 0 an edge is admissible
 // (slack 0, Eq. 2 with equality) iff  cbar(b,a) + k(a) == y(b) - 1.  Both
@@ -288,6 +290,7 @@ struct Smem {
     int fbest[kFastRows];     // fast rounds: each row's lowest candidate
     int4 frow[kFastRows];     // ... (row, scan start, target, 1 if it scanned)
     int nfl[2], nql[2];
+    int nleft, far;           // first rounds: rows with long scans; 1 if they were many (no near_scans then)
     int njob, ndon, don_base;
     int had_prop, nonfirst, nf_delta, donated;
     unsigned long long bytes;
@@ -659,12 +662,16 @@ __device__ __forceinline__ int warp_scan_slot(const unsigned char *slot, const C
 // while 32 jobs cover the CTA) and one 16-byte load per lane and step, at most
 // kNearSteps steps; the warp scans what is left of a row that needs more.
 // Only for floor(1/eps) <= kNearMaxK: at eps = 0.02 a later scan already
-// examines some 400 entries, and the whole solve was 0.5 % slower with it.
+// examines some 400 entries, and the whole solve was 0.5 % slower with it.  And
+// only if at most a quarter of the CTA's rows examined over kFarCells entries in
+// the phase's first round (costs that are rarely small, as between images, have
+// long scans at any eps).
 // n = 10,000, eps = 0.1 (147 rounds, 30 rows per CTA, 75 entries per scan), where
 // the slots copied whole row tails: solve 1084 -> 868 us; n = 6000 634 -> 561 us,
 // n = 10,000 at eps = 0.3 7.9 -> 6.3 ms, n = 1000 (3 rows per CTA) unchanged.
 // ---------------------------------------------------------------------------
 constexpr int kNearSteps = 4;
+constexpr int kFarCells = 1024;
 constexpr long long kNearMaxK = 20;
 
 template <class CB, bool F7>
@@ -747,7 +754,7 @@ __device__ __forceinline__ void run_jobs(Smem &s, const Lists &g, const Params &
     // slots (up to 16 rows in flight instead of rows_per_group); the choice is
     // this CTA's own.  The slot scan reads every unknown y(b) first (the
     // register scan reads it inside the row scan).
-    const bool near = !OFS && p.near && R > Rps && nq > rows_per_group;
+    const bool near = !OFS && p.near && R > Rps && nq > rows_per_group && !s.far;
     const bool via_slots = SL && !near && nq > rows_per_group;
     if (via_slots)
         for (int j = threadIdx.x; j < nq; j += blockDim.x)
@@ -850,6 +857,7 @@ __device__ __forceinline__ void run_jobs(Smem &s, const Lists &g, const Params &
             org = sp == p.nA ? 0 : sp;
         }
         cells += ex;
+        if (!OFS && p.near && R == Rps && ex > (unsigned)kFarCells) atomicAdd(&s.nleft, 1);
         if (a != 0x7FFFFFFF) {
             const unsigned long long old = atomicMax(p.prop + a, word_of(R, b));
             const unsigned t = tag_of(old);
@@ -894,6 +902,10 @@ __device__ __forceinline__ void run_jobs(Smem &s, const Lists &g, const Params &
         }
     }
     if (threadIdx.x == 0) {
+        if (p.near && R == Rps) {
+            s.far = 4 * s.nleft > nq ? 1 : 0;
+            s.nleft = 0;
+        }
         s.rows += (unsigned long long)nq;
         s.njob = 0;
         if (p.profile) {
@@ -1077,6 +1089,7 @@ k_phases(Params p, int warps_per_row, int rows_per_group) {
     if (threadIdx.x == 0) {
         s.nfl[0] = s.nfl[1] = s.nql[0] = s.nql[1] = 0;
         s.njob = s.ndon = 0;
+        s.nleft = s.far = 0;
         s.bytes = s.rows = s.cells = 0;
         s.err = 0;
         for (int i = 0; i < 4; ++i) s.cbar[i][0] = s.cbar[i][1] = 0;
