@@ -39,6 +39,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
+#include <stddef.h>
 #include <stdlib.h>
 #include <string.h>
 
@@ -182,6 +183,15 @@ __device__ __forceinline__ int phase_offset(long long phase1, int b, int nA) {
     return (int)(x % (unsigned long long)nA);
 }
 
+// Thread t of n clears its words of the control block and writes the mark.
+// (As one thread's memset k_solo_init took 5.7 us instead of 1.9, k_init 3.6
+// instead of 2.7.)
+__device__ __forceinline__ void clear_ctl(Ctl *c, int t, int n) {
+    static_assert(sizeof(Ctl) % 4 == 0 && offsetof(Ctl, head) == 0, "cleared by words, the head first");
+    for (int i = t; i < (int)(sizeof(Ctl) / 4); i += n)
+        reinterpret_cast<int *>(c)[i] = i == (int)(offsetof(WsHead, magic) / 4) ? kWsMagic : 0;
+}
+
 // ---------------------------------------------------------------------------
 // k_init
 // ---------------------------------------------------------------------------
@@ -200,11 +210,7 @@ __global__ void k_init(Params p, int *match_b) {
     // every pool slot free (y = 0, see pool_take)
     unsigned long long *pool = reinterpret_cast<unsigned long long *>(p.pool);
     for (long long i = t0; i < 2ll * p.nB; i += stride) pool[i] = 0;
-    if (t0 == 0) {
-        Ctl *c = p.ctl;
-        memset(c, 0, sizeof(Ctl));
-        c->head.magic = kWsMagic;
-    }
+    clear_ctl(p.ctl, t0, stride);
 }
 
 // ---------------------------------------------------------------------------
@@ -1579,10 +1585,7 @@ __global__ void __launch_bounds__(32) k_cost(Params p, Src src, const int *match
 // ---------------------------------------------------------------------------
 constexpr int kSoloThreads = 512;
 
-__global__ void k_solo_init(Ctl *c) {
-    memset(c, 0, sizeof(Ctl));
-    c->head.magic = kWsMagic;
-}
+__global__ void k_solo_init(Ctl *c) { clear_ctl(c, threadIdx.x, blockDim.x); }  // one CTA
 
 // The matched costs that k_solo adds up, whatever their source.
 struct SoloCost {
@@ -2134,7 +2137,7 @@ pr_status launch_solve(Params &p, const CostSource &src, double eps, const Phase
     bool solo;
     use_cta(p, cfg.smem, cb8 ? 1 : 2, K, solo);
     const bool take_over = p.hand > 0 || p.mid != 0;
-    if (solo) k_solo_init<<<1, 1, 0, st>>>(p.ctl);
+    if (solo) k_solo_init<<<1, 256, 0, st>>>(p.ctl);
     else k_init<<<di.sms * 2, 256, 0, st>>>(p, row_to_col);
     PR_CUDA(cudaGetLastError());
     const long long groups = (long long)n_rows * (p.ldq >> 3);
