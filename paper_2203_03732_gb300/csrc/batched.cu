@@ -229,12 +229,21 @@ constexpr int kPointCtas = 3;  // CTAs of k_bpoints_quant per SM, by its registe
 template <int DIM, bool SQ, class CB>
 __global__ void __launch_bounds__(256, kPointCtas) k_bpoints_quant(const float *__restrict__ XA, const float *__restrict__ XB, int dim,
                                 const BDesc *__restrict__ d, int P, int total_rows,
-                                const unsigned *__restrict__ maxbits, EpsSplit e, CB *__restrict__ cb) {
+                                const unsigned *__restrict__ maxbits, EpsSplit e, CB *__restrict__ cb, WsHead *head) {
     const int lane = threadIdx.x & 31;
+    bool bad = false;
     point_tiles(d, P, total_rows, [&](int i, int r, int rows) {
         const BDesc D = d[i];
         const PointsScale ps = points_scale(maxbits[i], SQ, e);
         CB *out = cb + D.cb_off + (long long)(r - D.v_off) * D.ldq;
+        // A rounded cost that is no cost (NaN or infinite coordinates, an
+        // infinite largest distance) is reported, and stored as 0: the marker's
+        // low byte is the padding's, whose sums carry into real columns.
+        const auto checked = [&](float dist, uint32_t k) {
+            if (dist >= 0.0f && dist <= ps.M && k != 0xFFFFFFFFu) return k;
+            bad = true;
+            return 0u;
+        };
         if constexpr (DIM == 0) {
             for (int q = 0; q < rows; ++q)
                 for (int a = lane; a < D.ldq; a += 32) {
@@ -243,7 +252,7 @@ __global__ void __launch_bounds__(256, kPointCtas) k_bpoints_quant(const float *
                         const float dd =
                             dist_f32(XB + (long long)(r + q) * dim, XA + (long long)(D.v_off + a) * dim, dim, SQ);
                         const float c = ps.M > 0.0f ? __fdiv_rn(dd, ps.M) : 0.0f;
-                        h = quantise_fbits(__float_as_uint(c), e);
+                        h = checked(dd, quantise_fbits(__float_as_uint(c), e));
                     }
                     out[(long long)q * D.ldq + a] = (CB)h;
                 }
@@ -259,7 +268,7 @@ __global__ void __launch_bounds__(256, kPointCtas) k_bpoints_quant(const float *
                     float sq[4];
                     uint32_t h[4];
                     sq_group4<DIM>(xb[q], xa, sq);
-                    quantise_points<4>(sq, SQ, ps, e, h, [](float, uint32_t k) { return k; });
+                    quantise_points<4>(sq, SQ, ps, e, h, checked);
                     if (a + 4 > D.n) {
 #pragma unroll
                         for (int j = 0; j < 4; ++j)
@@ -274,6 +283,7 @@ __global__ void __launch_bounds__(256, kPointCtas) k_bpoints_quant(const float *
             }
         }
     });
+    if (bad) record_error(head, PR_ERR_INVALID);
 }
 
 // ---------------------------------------------------------------------------
@@ -294,6 +304,19 @@ struct BatchCost {
     }
 };
 
+// Outputs of a problem that is not solved, because an error was recorded (an
+// asynchronous loss and its gradients are then NaN, not what the buffers held).
+__device__ void write_unsolved(const BParams &p, const BDesc &D, int pi) {
+    for (int i = threadIdx.x; i < D.n; i += blockDim.x) {
+        p.row_to_col[D.v_off + i] = p.col_to_row[D.v_off + i] = kUnsolved;
+        p.y_row[D.v_off + i] = p.y_col[D.v_off + i] = 0;
+    }
+    if (threadIdx.x == 0) {
+        p.costs[pi] = __longlong_as_double(0x7FF8000000000000ll);
+        p.phases[pi] = 0;
+    }
+}
+
 // CTAs per SM the registers are held to: 128 registers a thread at 128 and 256
 // threads, so that 4 and 2 CTAs fit (the compiler takes 172 otherwise, and one
 // CTA of 256 threads sat alone on an SM: 512 problems of up to 2048 rows 2.69
@@ -308,7 +331,7 @@ template <int THREADS, int UNROLL, class CB, bool F7>
 __global__ void __launch_bounds__(THREADS, kSolveCtas<THREADS>) k_bsolve(BParams p) {
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ CtaShared s;
-    __shared__ int cur_problem;
+    __shared__ int cur_problem, stopped;
     __shared__ double part[THREADS > kCostSums ? THREADS : kCostSums];
     const CtaLayout L(p.n_max, p.n_max);
     const CtaState<CB> state(dyn, L);
@@ -317,16 +340,19 @@ __global__ void __launch_bounds__(THREADS, kSolveCtas<THREADS>) k_bsolve(BParams
 
     for (;;) {
         if (threadIdx.x == 0) {
-            int t = (int)atomicAdd(&p.ctl->queue, 1u);
-            if (ld_relaxed_s32(&p.ctl->head.abort)) t = p.nprob;  // stop after an error
-            cur_problem = t;
+            cur_problem = (int)atomicAdd(&p.ctl->queue, 1u);
+            stopped = ld_relaxed_s32(&p.ctl->head.abort);  // nothing is solved after an error
         }
         __syncthreads();
-        const int t = cur_problem;
-        __syncthreads();  // every thread has read cur_problem before it changes
+        const int t = cur_problem, stop = stopped;
+        __syncthreads();  // every thread has read them before they change
         if (t >= p.nprob) break;
         const int pi = p.order[t];
         const BDesc D = p.desc[pi];
+        if (stop) {
+            write_unsolved(p, D, pi);
+            continue;
+        }
         const CB *cb = static_cast<const CB *>(p.cb) + D.cb_off;
         CtaCounts c = {0, 0, 0, 0, false};
         cta_init(s, state, D.n, D.n, D.ldq);
@@ -340,6 +366,7 @@ __global__ void __launch_bounds__(THREADS, kSolveCtas<THREADS>) k_bsolve(BParams
         }
         if (c.failed) {
             if (threadIdx.x == 0) record_error(&p.ctl->head, PR_ERR_NO_CONVERGENCE);
+            write_unsolved(p, D, pi);
             __syncthreads();
             continue;
         }
@@ -499,8 +526,9 @@ pr_status run_batched(const Source &src, int32_t P, const int32_t *n_host, doubl
         PR_CUDA(cudaLaunchKernel(kmax, dim3(std::min(di.sms * 4, tiles)), dim3(256), amax, 0, st));
         const unsigned *cmx_ = d_max;
         void *cbp_ = d_cb;
+        WsHead *head_ = &ctl->head;
         void *aq[] = {(void *)&xa_, (void *)&xb_, (void *)&dim_, (void *)&dd_, (void *)&P_,
-                      (void *)&rows_, (void *)&cmx_, (void *)&e, (void *)&cbp_};
+                      (void *)&rows_, (void *)&cmx_, (void *)&e, (void *)&cbp_, (void *)&head_};
         PR_CUDA(cudaLaunchKernel(kq, dim3(std::min(di.sms * kPointCtas, tiles)), dim3(256), aq, 0, st));
     } else if (src.dt == PR_F64) {
         if (cb8)
