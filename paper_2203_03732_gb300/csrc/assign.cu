@@ -1565,6 +1565,7 @@ __global__ void __launch_bounds__(32) k_cost(Params p, Src src, const int *match
     for (int b = v; b < p.nB; b += kFinThreads) acc = __dadd_rn(acc, src(b, match_b[b]));
     p.part[v] = acc;
     __threadfence();
+    __syncwarp();  // every lane's sum is stored before lane 0 counts the CTA
     unsigned last = 0;
     if (lane == 0) last = atomicAdd(&p.ctl->cost_done, 1u) == gridDim.x - 1 ? 1u : 0u;
     if (!__shfl_sync(0xFFFFFFFFu, last, 0)) return;
