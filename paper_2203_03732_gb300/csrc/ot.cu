@@ -373,6 +373,7 @@ __device__ __forceinline__ bool list_add_hi(const OParams &p, int a, int b, int 
         }
         __syncwarp();
     }
+    __syncwarp();  // every lane has read the list's length (an empty list has no steps above)
     if (lane == 0) {
         p.eb[off + pos] = b;
         p.elo[off + pos] = 0;
@@ -473,6 +474,7 @@ __device__ __forceinline__ unsigned ot_round(const OParams &p, unsigned R, unsig
             km = p.kmin[at];
             g = min(rb, left);
             rb -= g;
+            __syncwarp();  // every lane has read the copies left
             if (lane == 0) {
                 st_relaxed_u64(p.avail + at, ((unsigned long long)(R - 1) << 32) | (unsigned)(left - g));
                 p.clo[at] -= g;
