@@ -51,6 +51,7 @@
 #include "quantise.cuh"
 #include "points.cuh"
 #include "cta_solve.cuh"
+#include "cta_choice.cuh"
 
 namespace prot {
 namespace {
@@ -74,7 +75,6 @@ constexpr int kListSm = 1024;             // proposal-list entries kept in share
 constexpr int kKeepMax = 16;              // rows a CTA may keep for its next phase
 constexpr int kFastRows = 4;              // rows of a CTA in a fast round (fast_scan)
 constexpr int kFastUnroll = 5;            // 16-byte loads in flight per lane there: 10 KB over 4 warps
-constexpr int kBatch = 256;               // items turned into scan jobs at a time
 constexpr int kMaxGrid = 1023;            // barrier payload field width
 constexpr unsigned kMidRounds = 16;       // rounds of a phase before k_solo may take over inside it
 
@@ -1062,11 +1062,9 @@ k_phases(Params p, int warps_per_row, int rows_per_group) {
     // Every free row goes to the pool, which deals them out evenly, and the
     // rounds of few rows are fast ones; the forms without them keep up to a
     // register group's worth of rows when rows are short.
-    const int keep = (OFS || CL || p.nB > kBatch * (int)G) && rows_per_group > 2 ? min(rows_per_group - 1, kKeepMax) : 0;
-    // Every next-phase row goes to the pool and no CTA takes more than kBatch
-    // rows in a round (so its donations of a round fit s.don): the barrier
-    // places the donations (grid_sync_pool).
-    const bool place_at_barrier = !CL && keep == 0 && p.nB <= kBatch * (int)G;
+    const int keep = (OFS || CL || !all_to_pool(p.nB, (int)G)) && rows_per_group > 2 ? min(rows_per_group - 1, kKeepMax) : 0;
+    // The barrier places the donations (grid_sync_pool).
+    const bool place_at_barrier = !CL && keep == 0 && all_to_pool(p.nB, (int)G);
     Lists g;
     int *base = p.lists + (size_t)cta * p.list_stride;
     g.ql[0] = reinterpret_cast<int4 *>(base);
@@ -1951,55 +1949,12 @@ bool use_cluster(const PhaseCfg &cfg, int nslots, int n_rows, long long K, int r
     return rule == PR_RULE_OFFSET && n_rows <= kClusterMaxRows && K > kClusterMinK;
 }
 
-// Small problems.  A round of the grid costs about 4.3 us whatever it does (a
-// grid barrier and four or five dependent L2 trips); on one CTA with its
-// state in shared memory it costs 0.9 us with a few rows, and grows with the
-// rows, since one SM scans them all.  So one CTA runs problems of up to
-// kSoloMaxRows rows from the start, and for larger ones the grid runs the
-// first, crowded phases and one CTA the rest, from the first phase with at
-// most kHandRows free rows (fewer with long rows: kHandBytes of rounded costs
-// in all).  Where T is not below that, the grid runs alone.  Solve time, ms,
-// eps = 0.01 / 0.003, one CTA / take-over / grid: n = 300: 0.46 / 0.47 / 1.44,
-// 12.6 / 12.9 / 54; n = 1000: 1.61 / 1.60 / 3.93, 8.8 / 8.6 / 24.7; n = 2000:
-// 1.70 / 1.44 / 2.23, 16.4 / 14.3 / 30.6; n = 4000: 3.85 / 2.53 / 2.79, 36 /
-// 24.0 / 27.4; 1000 x 1500: 0.23 / 0.13 / 0.17, 0.72 / 0.41 / 0.63.  Half or
-// twice the rows or bytes was slower; rows past kHandRowBytes as well (n =
-// 6000 in 16 bits: 43.0 against 41.8).
-constexpr int kSoloMaxRows = 384;
-constexpr int kHandRows = 64, kHandBytes = 256 * 1024, kHandRowBytes = 8192;
-// At floor(1/eps) <= kNearMaxK most of a solve can be one phase of a hundred
-// rounds in which hundreds of rows lose the same columns (squared distances, n
-// = 1000, eps = 0.1: 131 rounds of 464 rows).  The grid's rounds cost 4.3 us,
-// one CTA's 2.3 us at 512 to 1024 rows, so one CTA takes over inside a phase
-// that has lasted kMidRounds rounds: that solve 574 -> 347 us, n = 1500 855 -> 552
-// us, n = 1000 at eps = 0.3 1545 -> 701 us.  (A problem of 20 rounds is faster on
-// the grid: n = 1000, Euclidean, 122 us against 153 us on one CTA; at n = 2000
-// such a problem is 8 % slower with the take-over, 228 against 210 us.)
-constexpr int kMidRows = 1536;
-
-// Whether one CTA runs the problem from the start (solo), takes over from the
-// grid once at most p.hand rows are free (0: never), or inside a long phase
-// (p.mid).
-void use_cta(Params &p, size_t smem_max, int key_bytes, long long K, bool &solo) {
-    solo = false;
-    p.hand = p.mid = 0;
-    if ((p.rule != PR_RULE_LOWEST && p.rule != PR_RULE_SEQUENTIAL) || p.profile || p.nA > kCtaMaxCols) return;
-    if (CtaLayout(p.nB, p.nA).total(key_bytes) + kCtaStaticSmem > smem_max) return;
-    const char *m = getenv("PR_PHASE_MODE");
-    if (m && (strcmp(m, "grid") == 0 || strcmp(m, "cluster") == 0)) return;
-    const bool seq = p.rule == PR_RULE_SEQUENTIAL;
-    if (m ? strcmp(m, "solo") == 0 : p.nB <= kSoloMaxRows && !seq) {
-        solo = true;
-        return;
-    }
-    // the sequential rule: half the bytes, and never from the start (ms, grid /
-    // take-over: n = 200, eps = 0.01 2.28 / 0.63, n = 1000, eps = 0.003 24.1 /
-    // 9.0, n = 2000, eps = 0.01 1.85 / 1.43; n = 4000, eps = 0.01 with 64 rows of
-    // 4 KB 2.10 / 2.26; n = 384, eps = 0.1 on one CTA alone 0.07 / 0.17)
-    const int row_bytes = p.ldq * key_bytes;
-    const int rows = std::min(kHandRows, (seq ? kHandBytes / 2 : kHandBytes) / row_bytes);
-    if (row_bytes <= kHandRowBytes && rows > p.T) p.hand = rows;
-    p.mid = !seq && K <= kNearMaxK && p.nB <= kMidRows;
+// Where one CTA runs the problem or takes it over (cta_choice.cuh).
+CtaChoice use_cta(const Params &p, size_t smem_max, int key_bytes, long long K, int ctas) {
+    if ((p.rule != PR_RULE_LOWEST && p.rule != PR_RULE_SEQUENTIAL) || p.profile || p.nA > kCtaMaxCols) return {};
+    if (CtaLayout(p.nB, p.nA).total(key_bytes) + kCtaStaticSmem > smem_max) return {};
+    return choose_cta(p.rule == PR_RULE_SEQUENTIAL, p.nB, p.ldq * key_bytes, p.T, K <= kNearMaxK, ctas,
+                      getenv("PR_PHASE_MODE"));
 }
 
 // Row scans of the grid form: a CTA with more jobs than one register group
@@ -2135,9 +2090,10 @@ pr_status launch_solve(Params &p, const CostSource &src, double eps, const Phase
     const bool f7 = cb8 && K <= kMaxCbar7;  // and cbar + key < 256 on every real column
 
     const DeviceInfo &di = device_info();
-    bool solo;
-    use_cta(p, cfg.smem, cb8 ? 1 : 2, K, solo);
-    const bool take_over = p.hand > 0 || p.mid != 0;
+    const CtaChoice cta = use_cta(p, cfg.smem, cb8 ? 1 : 2, K, cfg.grid);
+    const bool solo = cta.solo, take_over = cta.hand > 0 || cta.mid;
+    p.hand = cta.hand;
+    p.mid = cta.mid ? 1 : 0;
     if (solo) k_solo_init<<<1, 256, 0, st>>>(p.ctl);
     else k_init<<<di.sms * 2, 256, 0, st>>>(p, row_to_col);
     PR_CUDA(cudaGetLastError());
