@@ -1400,9 +1400,9 @@ k_phases(Params p, int warps_per_row, int rows_per_group) {
         }
     }
 done:
-    if (cells) atomicAdd(&s.cells, cells);
-    if (fast_bytes) atomicAdd(&s.bytes, fast_bytes);
-    if (fast_rows) atomicAdd(&s.rows, fast_rows);
+    warp_count(&s.cells, cells);
+    warp_count(&s.bytes, fast_bytes);
+    warp_count(&s.rows, fast_rows);
     __syncthreads();
     if (threadIdx.x == 0) {
         if (s.bytes) atomicAdd(&ctl->bytes, s.bytes);

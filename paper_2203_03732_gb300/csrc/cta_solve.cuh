@@ -460,9 +460,9 @@ __device__ __forceinline__ void cta_phases(CtaShared &s, const CtaState<CB> &st,
         cur = nxt;
     }
     out.free_at_stop = nf;
-    if (my_cells) atomicAdd(&s.cells, my_cells);
-    if (my_bytes) atomicAdd(&s.bytes, my_bytes);
-    if (my_rows) atomicAdd(&s.rows, my_rows);
+    warp_count(&s.cells, my_cells);
+    warp_count(&s.bytes, my_bytes);
+    warp_count(&s.rows, my_rows);
     __syncthreads();
 }
 
@@ -562,8 +562,8 @@ __device__ __forceinline__ void cta_seq_phases(CtaShared &s, const CtaState<CB> 
     }
     out.rounds = out.phases;
     out.free_at_stop = nf;
-    if (my_cells) atomicAdd(&s.cells, my_cells);
-    if (my_bytes) atomicAdd(&s.bytes, my_bytes);
+    warp_count(&s.cells, my_cells);
+    warp_count(&s.bytes, my_bytes);
     __syncthreads();
 }
 
