@@ -678,7 +678,6 @@ __device__ __forceinline__ int warp_scan_slot(const unsigned char *slot, const C
 // ---------------------------------------------------------------------------
 constexpr int kNearSteps = 4;
 constexpr int kFarCells = 1024;
-constexpr long long kNearMaxK = 20;
 
 template <class CB, bool F7>
 __device__ __forceinline__ void near_scans(Smem &s, const Params &p, const CB *ks, const unsigned *tk, int nq) {
@@ -1953,7 +1952,7 @@ bool use_cluster(const PhaseCfg &cfg, int nslots, int n_rows, long long K, int r
 CtaChoice use_cta(const Params &p, size_t smem_max, int key_bytes, long long K, int ctas) {
     if ((p.rule != PR_RULE_LOWEST && p.rule != PR_RULE_SEQUENTIAL) || p.profile || p.nA > kCtaMaxCols) return {};
     if (CtaLayout(p.nB, p.nA).total(key_bytes) + kCtaStaticSmem > smem_max) return {};
-    return choose_cta(p.rule == PR_RULE_SEQUENTIAL, p.nB, p.ldq * key_bytes, p.T, K <= kNearMaxK, ctas,
+    return choose_cta(p.rule == PR_RULE_SEQUENTIAL, p.nB, p.nA, p.ldq * key_bytes, p.T, K, ctas,
                       getenv("PR_PHASE_MODE"));
 }
 

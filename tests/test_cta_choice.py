@@ -11,8 +11,9 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 
 SRC = """
 #include "cta_choice.cuh"
-extern "C" void choose(int seq, int n_rows, int row_bytes, int T, int coarse, int ctas, const char *mode, int *out) {
-    const prot::CtaChoice c = prot::choose_cta(seq, n_rows, row_bytes, T, coarse, ctas, mode);
+extern "C" void choose(int seq, int n_rows, int n_cols, int row_bytes, int T, int K, int ctas, const char *mode,
+                       int *out) {
+    const prot::CtaChoice c = prot::choose_cta(seq, n_rows, n_cols, row_bytes, T, K, ctas, mode);
     out[0] = c.solo; out[1] = c.hand; out[2] = c.mid;
 }
 """
@@ -30,7 +31,7 @@ def choose(tmp_path_factory):
         K = int(1 / eps)
         row_bytes = (n_cols + 31) // 32 * 32 * (1 if K <= 252 else 2)
         out = (ctypes.c_int * 3)()
-        L.choose(int(seq), n_rows, row_bytes, int(eps * n_rows), int(K <= 20), ctas, mode, out)
+        L.choose(int(seq), n_rows, n_cols, row_bytes, int(eps * n_rows), K, ctas, mode, out)
         return dict(solo=bool(out[0]), hand=out[1], mid=bool(out[2]))
     return f
 
@@ -55,3 +56,13 @@ def test_lines_of_the_rule(choose):
     assert not choose(1536, 1536, 0.04)["mid"]  # floor(1/eps) > 20
     assert choose(300, 300, 0.1, mode=b"grid") == dict(solo=False, hand=0, mid=False)
     assert choose(4000, 4000, 0.01, mode=b"solo")["solo"]
+
+
+@pytest.mark.parametrize("n_rows,n_cols,eps,solo", [
+    (64, 8000, 0.005, True), (64, 8000, 0.003, False), (32, 8000, 0.003, True),  # 512 KB of rounded costs
+    (384, 8000, 0.05, True), (384, 8000, 0.04, False), (65, 8000, 0.02, True), (200, 8000, 0.02, True),
+    (201, 8000, 0.02, False), (65, 8000, 0.01, False), (384, 8000, 0.003, False), (300, 7000, 0.01, False),
+    (384, 512, 0.01, True), (384, 513, 0.01, False), (300, 450, 0.003, True), (300, 600, 0.003, False)])
+def test_one_cta_from_the_start(choose, n_rows, n_cols, eps, solo):
+    """Wide problems whose crowded phases one SM would scan alone go to the grid."""
+    assert choose(n_rows, n_cols, eps)["solo"] == solo
