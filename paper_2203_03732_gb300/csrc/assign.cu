@@ -933,7 +933,7 @@ __device__ __forceinline__ void run_jobs(Smem &s, const Lists &g, const Params &
 // 10,000, eps = 0.01 4.18 -> 3.56, eps = 0.005 14.2 -> 12.1; n = 6000, eps = 0.01
 // 3.75 -> 2.79 (with every row to the pool, which it kept from its CTA's next
 // phase before).  Rounds with more rows per CTA pay 0.16 us for the longer
-// code (n = 10,000, eps = 0.1, 147 rounds: 863 -> 887 us).
+// code (crowded_rounds).
 // ---------------------------------------------------------------------------
 template <class CB>
 struct FastRow {
@@ -1042,8 +1042,8 @@ __host__ __device__ inline size_t slots_offset(int ldq, int key_bytes) {
 // CL: the launch is one thread-block cluster (barriers through distributed
 // shared memory) instead of a cooperative grid.  SL: a CTA whose jobs exceed
 // one register group scans them from per-warp shared-memory slots filled by
-// bulk copies (always with CL).
-template <class CB, bool CL, bool SL, bool F7, bool OFS>
+// bulk copies (always with CL).  FAST: rounds of few rows are fast rounds.
+template <class CB, bool CL, bool SL, bool F7, bool OFS, bool FAST = !CL && !OFS>
 __global__ void __launch_bounds__(kThreads, 1)
 k_phases(Params p, int warps_per_row, int rows_per_group) {
     extern __shared__ __align__(16) unsigned char dyn[];
@@ -1107,7 +1107,7 @@ k_phases(Params p, int warps_per_row, int rows_per_group) {
     // started and zeroed them.
     if (CL) cluster_barrier_hw();
 
-    const bool fast_ok = !OFS && place_at_barrier && !p.profile;
+    const bool fast_ok = FAST && place_at_barrier && !p.profile;
     unsigned long long fast_bytes = 0, fast_rows = 0;  // this thread's, added up at exit
     unsigned gen = 0;
     unsigned R = 0;  // global round counter (round tags)
@@ -1823,16 +1823,17 @@ struct PhaseCfg {
     size_t smem = 0;
 };
 
-template <class CB, bool CL, bool SL, bool F7, bool OFS = false>
+template <class CB, bool CL, bool SL, bool F7, bool OFS = false, bool FAST = !CL && !OFS>
 pr_status set_phase_attrs(size_t smem) {
-    PR_CUDA(cudaFuncSetAttribute(k_phases<CB, CL, SL, F7, OFS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    if (CL) PR_CUDA(cudaFuncSetAttribute(k_phases<CB, CL, SL, F7, OFS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    PR_CUDA(cudaFuncSetAttribute(k_phases<CB, CL, SL, F7, OFS, FAST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (CL) PR_CUDA(cudaFuncSetAttribute(k_phases<CB, CL, SL, F7, OFS, FAST>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     return PR_OK;
 }
 
 // The phase kernel for the storage type (cb8: bytes), the form (cl: one
 // cluster, sl: row slots), the byte pre-test (f7: floor(1/eps) <= 125) and
-// the step I rule (ofs: PR_RULE_OFFSET).
+// the step I rule (ofs: PR_RULE_OFFSET).  crowded: the form without fast rounds
+// (crowded_rounds), in bytes with slots.
 template <bool OFS>
 const void *phase_kernel_of(bool cb8, bool cl, bool sl, bool f7) {
     if (!cb8)
@@ -1847,7 +1848,8 @@ const void *phase_kernel_of(bool cb8, bool cl, bool sl, bool f7) {
               : sl ? (const void *)k_phases<uint8_t, false, true, false, OFS>
                    : (const void *)k_phases<uint8_t, false, false, false, OFS>;
 }
-const void *phase_kernel(bool cb8, bool cl, bool sl, bool f7, bool ofs) {
+const void *phase_kernel(bool cb8, bool cl, bool sl, bool f7, bool ofs, bool crowded = false) {
+    if (crowded && cb8 && !cl && sl && f7 && !ofs) return (const void *)k_phases<uint8_t, false, true, true, false, false>;
     return ofs ? phase_kernel_of<true>(cb8, cl, sl, f7) : phase_kernel_of<false>(cb8, cl, sl, f7);
 }
 
@@ -1896,6 +1898,7 @@ pr_status phase_cfg(PhaseCfg &cfg) {
     if (rc == PR_OK) rc = set_phase_attrs<uint8_t, false, false, true>(smem);
     if (rc == PR_OK) rc = set_phase_attrs<uint8_t, false, true, true>(smem);
     if (rc == PR_OK) rc = set_phase_attrs<uint8_t, true, true, true>(smem);
+    if (rc == PR_OK) rc = set_phase_attrs<uint8_t, false, true, true, false, false>(smem);
     if (rc == PR_OK) rc = set_phase_attrs<uint16_t, false, false, false, true>(smem);
     if (rc == PR_OK) rc = set_phase_attrs<uint16_t, false, true, false, true>(smem);
     if (rc == PR_OK) rc = set_phase_attrs<uint16_t, true, true, false, true>(smem);
@@ -1947,6 +1950,13 @@ bool use_cluster(const PhaseCfg &cfg, int nslots, int n_rows, long long K, int r
     if (m && strcmp(m, "cluster") == 0) return true;
     return rule == PR_RULE_OFFSET && n_rows <= kClusterMaxRows && K > kClusterMinK;
 }
+
+// Where nearly every round has more rows than the CTAs' fast rounds take, the
+// phase loop is compiled without them (shorter code).  us, without / with:
+// n = 10,000, eps = 0.1 927 / 948, image-shaped 413 / 420 at eps = 0.1, 10,185 /
+// 10,409 at 0.75; n = 6000, eps = 0.1 504 / 519; n = 3000 272 / 277, image-shaped
+// 138 / 135; n = 2000 202 / 203; eps = 0.02 n = 4000 867 / 738.
+bool crowded_rounds(int n_rows, long long K) { return K <= kNearMaxK && n_rows > 4096; }
 
 // Where one CTA runs the problem or takes it over (cta_choice.cuh).
 CtaChoice use_cta(const Params &p, size_t smem_max, int key_bytes, long long K, int ctas) {
@@ -2187,7 +2197,7 @@ pr_status launch_solve(Params &p, const CostSource &src, double eps, const Phase
         Params pc = p;
         void *args[] = {(void *)&pc, (void *)&warps_per_row, (void *)&rows_per_group};
         const bool sl = use_slots_in_grid(p.nslots);
-        const void *fn = phase_kernel(cb8, false, sl, f7, p.rule != 0);
+        const void *fn = phase_kernel(cb8, false, sl, f7, p.rule != 0, crowded_rounds(n_rows, K));
         const size_t smem = sl ? slots_offset(p.ldq, kb) + (size_t)p.nslots * p.slot_bytes : smem_bytes(p.ldq, kb);
         PR_CUDA(cudaLaunchCooperativeKernel(fn, dim3(cfg.grid), dim3(kThreads), args, smem, st));
     }

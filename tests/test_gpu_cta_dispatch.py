@@ -48,3 +48,10 @@ def test_one_cta_from_the_start(prot, nB, nA, eps, one):
 def test_around_the_take_overs(prot, nB, nA, eps, squared):
     A, B = W.points_uniform(nA, nB, 2, 23)
     assert solve(prot, W.pairwise_cost(A, B, squared=squared), eps)["loop_ctas"] > 1
+
+
+@pytest.mark.parametrize("nB,nA", [(4096, 4096), (4097, 4100)])
+@pytest.mark.parametrize("eps", [0.1, 0.05, 0.04])
+def test_phase_loop_with_and_without_fast_rounds(prot, nB, nA, eps):
+    """floor(1/eps) <= 20 and more than 4096 rows: the loop without them."""
+    solve(prot, W.assignment_euclid_2d(nB, 31, n_a=nA), eps)
