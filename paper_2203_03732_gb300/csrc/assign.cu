@@ -292,11 +292,16 @@ struct Smem {
     int job_tgt[kBatch];
     int job_best[kBatch];
     int2 don[kBatch];         // pool entries given to the pool in this batch
-    int best[kWarps];
-    int fbest[kFastRows];     // fast rounds: each row's lowest candidate
-    int4 frow[kFastRows];     // ... (row, scan start, target, 1 if it scanned)
+    union {
+        int best[kWarps];      // run_jobs: each register group's lowest candidate
+        int fbest[kFastRows];  // fast rounds: each row's lowest candidate
+    };
+    union {
+        unsigned long long cbar[4][2];  // cluster mode: this CTA's copy of the barrier slots
+        int4 frow[kFastRows];           // fast rounds: (row, scan start, target, 1 if it scanned)
+    };
     int nfl[2], nql[2];
-    int nleft, far;           // first rounds: rows with long scans; 1 if they were many (no near_scans then)
+    int nleft;                // first rounds: rows with long scans
     int njob, ndon, don_base;
     int had_prop, nonfirst, nf_delta, donated;
     unsigned long long bytes;
@@ -304,10 +309,12 @@ struct Smem {
     unsigned long long cells;
     unsigned long long pub, pub2;
     unsigned long long pacc[4];  // profile: build, scan, proposal, tail ns of this round
-    unsigned long long cbar[4][2];  // cluster mode: this CTA's copy of the barrier slots
     unsigned long long mbar[kWarps];  // cluster mode: completion of each warp's row copy
     int err;
+    int far;                  // 1 if the rows with long scans were many (no near_scans in this phase)
 };
+// The keys share the space: this size gives the largest n_cols, 89,808.
+static_assert(sizeof(Smem) <= 41600, "n_cols up to 89,808");
 
 struct Lists {
     int4 *ql[2];  // global overflow of ql
@@ -2310,7 +2317,7 @@ pr_status assign_common(const CostSource &src, int32_t n_rows, int32_t n_cols, d
     if (smem_bytes(L.ldq) > cfg.smem)
         // each column costs 2 bytes of key copy and 1/8 byte of taken set
         return fail(PR_ERR_INVALID, "%s: n_cols = %d exceeds the shared-memory key copy (max %d)", who,
-                    n_cols, (int)((cfg.smem - smem_bytes(0)) * 8 / 17) & ~31);
+                    n_cols, (int)((cfg.smem - smem_bytes(0)) * 8 / 17) & ~15);
     if (!ws || ((uintptr_t)ws & 255) || ws_bytes < L.total)
         return fail(PR_ERR_WORKSPACE, "%s: workspace NULL, not 256-byte aligned or < %zu bytes", who,
                     L.total);
