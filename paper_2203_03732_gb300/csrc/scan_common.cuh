@@ -28,6 +28,7 @@ struct EpsSplit {
     int ee;
     float inv;
     float win;  // an estimate within win of an integer takes the exact test
+    float low;  // 0.25 eps: costs below it round to 0
 };
 
 // The FP32 estimate q of c / eps (c truncated to 24 significant bits:
@@ -44,6 +45,7 @@ inline EpsSplit make_eps_split(double eps) {  // eps normal, in (0, 1)
     e.inv = (float)(1.0 / eps);
     const double w = (floor(1.0 / eps) + 1.0) * ldexp(1.0, -21);
     e.win = (float)(w < 0.015625 ? w : 0.015625);
+    e.low = (float)(0.25 * eps);
     return e;
 }
 
@@ -122,32 +124,38 @@ __device__ __forceinline__ uint32_t quantise_fbits(uint32_t fb, const EpsSplit &
 }
 
 // ---------------------------------------------------------------------------
-// Eq. (1) for a group of N values: 7 (FP32) to 9 (FP64) instructions each on
+// Eq. (1) for a group of N values: 8 (FP32) to 13 (FP64) instructions each on
 // the way that nearly all take, against about 25 for quantise_bits one value
 // at a time, which bound the rounding kernels by instructions, not memory.
 //
 // t = 2^23 + v * scale rounded down has floor(v * scale) in its low bits (the
 // sum's unit is 1, and the product is not rounded first); d = v * scale -
 // floor - 1/2 tells how near an integer the estimate is.  A value whose |d|
-// is within `near` of 1/2, or whose bits lie outside the range that the
-// estimate covers, is settled by `exact(j)`; one test covers the group.
+// is within `near` of 1/2 is settled by `settle(j, m)`, m >= 1 the integer
+// nearest the estimate; a group with a value outside the range that the
+// estimate covers goes to `exact(j)` value by value; one test covers both.
+// Values below low (scale * low = 1/4) are taken as low: their floor is 0,
+// and exact zeros, common in real costs, stay on the short way.
 // Only the low 8 or 16 bits of h[j] are the result.
 // ---------------------------------------------------------------------------
-template <int N, class Exact>
-__device__ __forceinline__ void floor_group(const float (&v)[N], float scale, float near, bool out_of_range,
-                                            uint32_t (&h)[N], const Exact &exact) {
+template <int N, class Exact, class Settle>
+__device__ __forceinline__ void floor_group(const float (&v)[N], float scale, float low, float near, bool out_of_range,
+                                            uint32_t (&h)[N], const Exact &exact, const Settle &settle) {
     float d[N], far = 0.0f;
 #pragma unroll
     for (int j = 0; j < N; ++j) {
-        const float t = __fmaf_rd(v[j], scale, 8388608.0f);
-        d[j] = __fmaf_rn(v[j], scale, __fsub_rn(8388607.5f, t));  // 2^23 - 1/2 - t is exact
+        const float x = fmaxf(v[j], low);
+        const float t = __fmaf_rd(x, scale, 8388608.0f);
+        d[j] = __fmaf_rn(x, scale, __fsub_rn(8388607.5f, t));  // 2^23 - 1/2 - t is exact
         far = fmaxf(far, fabsf(d[j]));
         h[j] = __float_as_uint(t);
     }
     if (out_of_range || !(far <= 0.5f - near)) {
 #pragma unroll
-        for (int j = 0; j < N; ++j)
-            if (out_of_range || !(fabsf(d[j]) <= 0.5f - near)) h[j] = exact(j);
+        for (int j = 0; j < N; ++j) {
+            if (out_of_range) h[j] = exact(j);
+            else if (!(fabsf(d[j]) <= 0.5f - near)) h[j] = settle(j, (h[j] & 0xFFFFu) + (d[j] > 0.0f ? 1u : 0u));
+        }
     }
 }
 
@@ -158,34 +166,53 @@ __device__ __forceinline__ void quantise_group(const float (&c)[N], const EpsSpl
     uint32_t top = 0;
 #pragma unroll
     for (int j = 0; j < N; ++j) top = max(top, __float_as_uint(c[j]));
-    floor_group<N>(c, e.inv, e.win, top > 0x3F800000u, h, [&](int j) {
-        const uint32_t q = quantise_fbits(__float_as_uint(c[j]), e);
-        if (q == 0xFFFFFFFFu) bad = true;
-        return q == 0xFFFFFFFFu ? 0u : q;
-    });
+    floor_group<N>(
+        c, e.inv, e.low, e.win, top > 0x3F800000u, h,
+        [&](int j) {
+            const uint32_t q = quantise_fbits(__float_as_uint(c[j]), e);
+            if (q == 0xFFFFFFFFu) bad = true;
+            return q == 0xFFFFFFFFu ? 0u : q;
+        },
+        [&](int j, uint32_t m) {
+            const uint32_t fb = __float_as_uint(c[j]);
+            return ge_multiple((fb & 0x7FFFFFu) | 0x800000u, (int)(fb >> 23) - 150, m, e) ? m : m - 1u;
+        });
 }
 
-// FP64 costs: for 2^-127 <= c < 1 the exponent's low 7 bits and the mantissa's
+// FP64 costs: for 2^-126 <= c < 2 the exponent's low 7 bits and the mantissa's
 // leading 23 are those of c truncated to FP32 (relative error below 2^-23), so
 // with the rounding of 1/eps the error is below (floor(1/eps) + 1) * 1.5 *
-// 2^-23, inside e.win.  Everything else, 0 and 1 among it, is out of range.
+// 2^-23, inside e.win.  The high word of a smaller cost is raised to 2^-127's,
+// which gives a value below e.low.  Out of range: c > 1 (the bits less one,
+// compared from the high word down, reach 1's), NaN among it, or a sign bit.
+// (With 0 and 1 out of range, as at first, one of them sent all 8 values of a
+// group the long way: n = 10,000, 1 % ones at eps = 0.3, whole solve 191 ->
+// 241 us.)
 template <int N>
 __device__ __forceinline__ void quantise_group(const double (&c)[N], const EpsSplit &e, uint32_t (&h)[N], bool &bad) {
     float f[N];
-    uint32_t top = 0;
+    int top = 0;
+    uint32_t signs = 0;
 #pragma unroll
     for (int j = 0; j < N; ++j) {
         const unsigned long long b = (unsigned long long)__double_as_longlong(c[j]);
         const uint32_t hi = (uint32_t)(b >> 32), lo = (uint32_t)b;
-        f[j] = __uint_as_float(__funnelshift_l(lo, hi, 3) & 0x3FFFFFFFu);
-        top = max(top, hi - 0x38000000u);
+        f[j] = __uint_as_float(__funnelshift_l(lo, (uint32_t)max((int)hi, 0x38000000), 3) & 0x3FFFFFFFu);
+        top = max(top, (int)((b - 1ull) >> 32));
+        signs |= hi;
     }
-    floor_group<N>(f, e.inv, e.win, top >= 0x07F00000u, h, [&](int j) {
-        const unsigned long long b = (unsigned long long)__double_as_longlong(c[j]);
-        const uint32_t q = quantise_bits((uint32_t)(b >> 32), (uint32_t)b, e);
-        if (q == 0xFFFFFFFFu) bad = true;
-        return q == 0xFFFFFFFFu ? 0u : q;
-    });
+    floor_group<N>(
+        f, e.inv, e.low, e.win, top >= 0x3FF00000 || (int)signs < 0, h,
+        [&](int j) {
+            const unsigned long long b = (unsigned long long)__double_as_longlong(c[j]);
+            const uint32_t q = quantise_bits((uint32_t)(b >> 32), (uint32_t)b, e);
+            if (q == 0xFFFFFFFFu) bad = true;
+            return q == 0xFFFFFFFFu ? 0u : q;
+        },
+        [&](int j, uint32_t m) {
+            const unsigned long long b = (unsigned long long)__double_as_longlong(c[j]);
+            return ge_multiple((b & 0xFFFFFFFFFFFFFull) | (1ull << 52), (int)(b >> 52) - 1075, m, e) ? m : m - 1u;
+        });
 }
 
 // Costs from points: c = RN32(dist / M), dist the squared sum sq or its IEEE
@@ -196,7 +223,7 @@ __device__ __forceinline__ void quantise_group(const double (&c)[N], const EpsSp
 // (all values then, M is the same for all), and NaN.  exact_cost(dist, q) is
 // called with the exact way's distance and result and returns what to store.
 struct PointsScale {
-    float M, scale;
+    float M, scale, low;
     bool wide;
 };
 __device__ __forceinline__ PointsScale points_scale(uint32_t max_sq_bits, int squared, const EpsSplit &e) {
@@ -204,6 +231,7 @@ __device__ __forceinline__ PointsScale points_scale(uint32_t max_sq_bits, int sq
     p.M = squared ? __uint_as_float(max_sq_bits) : __fsqrt_rn(__uint_as_float(max_sq_bits));
     p.wide = !(p.M >= 1e-18f && p.M <= 1e18f);
     p.scale = p.wide ? 0.0f : __fdiv_rn(e.inv, p.M);
+    p.low = __fmul_rn(e.low, p.M);
     return p;
 }
 template <int N, class Cost>
@@ -217,11 +245,13 @@ __device__ __forceinline__ void quantise_points(const float (&sq)[N], int square
         if (!squared) asm("sqrt.approx.f32 %0, %1;" : "=f"(v[j]) : "f"(sq[j]));
         top = max(top, __float_as_uint(sq[j]));
     }
-    floor_group<N>(v, p.scale, 2.0f * e.win, p.wide || top >= 0x7F800000u, h, [&](int j) {
+    const auto exact = [&](int j) {
         const float d = squared ? sq[j] : __fsqrt_rn(sq[j]);
         const float c = p.M > 0.0f ? __fdiv_rn(d, p.M) : 0.0f;
         return exact_cost(d, quantise_fbits(__float_as_uint(c), e));
-    });
+    };
+    floor_group<N>(v, p.scale, p.low, 2.0f * e.win, p.wide || top >= 0x7F800000u, h, exact,
+                   [&](int j, uint32_t) { return exact(j); });
 }
 
 // Low bytes (16-bit halves) of four values as one stored word (pair).
