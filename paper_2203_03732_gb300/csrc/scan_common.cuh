@@ -49,19 +49,15 @@ inline EpsSplit make_eps_split(double eps) {  // eps normal, in (0, 1)
     return e;
 }
 
-// Exact test c >= m * eps for c = mc * 2^ec (mc < 2^53) and 1 <= m < 2^16,
-// in 128-bit integer arithmetic: both sides are brought to the smaller
-// exponent and compared.  Outside the shifts that fit in 128 bits the
-// answer follows from the exponents alone (c is normal, so 2^23 <= mc for
-// FP32 and 2^52 <= mc for FP64; 2^52 <= m * me < 2^69).
+// Exact test c >= m * eps for c = mc * 2^ec (2^23 <= mc < 2^53), 1 <= m < 2^16
+// and |c / eps - m| <= 1/16: the sign of 2 (mc 2^(ec - ee) - m me) in 64-bit
+// arithmetic mod 2^64.  As c is that near m eps, 2^(ec - ee) is between 1/2 and
+// 2^47 and the difference is below 2 me / 16 < 2^50.  About 12 instructions;
+// comparing two 128-bit numbers took 50, and in 16 copies per thread they thrashed
+// the instruction cache (n = 9999 FP32, 1 % ones at eps = 0.1, whole solve: 238 ->
+// 155 us; all costs multiples of eps, n = 10,000 FP64: 322 -> 207 us).
 __device__ __forceinline__ bool ge_multiple(unsigned long long mc, int ec, uint32_t m, const EpsSplit &e) {
-    const int d = ec - e.ee;
-    if (d > 74) return true;
-    if (d < -58) return false;
-    unsigned __int128 lhs = mc, rhs = (unsigned __int128)e.me * m;
-    if (d >= 0) lhs <<= d;
-    else rhs <<= -d;
-    return lhs >= rhs;
+    return (long long)((mc << (ec - e.ee + 1)) - ((e.me * m) << 1)) >= 0;
 }
 
 // Eq. (1) exactly: cbar = the largest k with k * eps <= c, for 0 <= c <= 1.
@@ -159,27 +155,21 @@ __device__ __forceinline__ void floor_group(const float (&v)[N], float scale, fl
     }
 }
 
-// FP32 costs.  The estimate's error is below (floor(1/eps) + 1) * 2^-23 (the
-// rounding of 1/eps), inside e.win.
+// The estimate's operand of each cost, and whether the group has a cost
+// outside the range that it covers.
+// FP32: the cost itself.  The estimate's error is below (floor(1/eps) + 1) *
+// 2^-23 (the rounding of 1/eps), inside e.win.
 template <int N>
-__device__ __forceinline__ void quantise_group(const float (&c)[N], const EpsSplit &e, uint32_t (&h)[N], bool &bad) {
+__device__ __forceinline__ bool group_operands(const float (&c)[N], float (&f)[N]) {
     uint32_t top = 0;
 #pragma unroll
-    for (int j = 0; j < N; ++j) top = max(top, __float_as_uint(c[j]));
-    floor_group<N>(
-        c, e.inv, e.low, e.win, top > 0x3F800000u, h,
-        [&](int j) {
-            const uint32_t q = quantise_fbits(__float_as_uint(c[j]), e);
-            if (q == 0xFFFFFFFFu) bad = true;
-            return q == 0xFFFFFFFFu ? 0u : q;
-        },
-        [&](int j, uint32_t m) {
-            const uint32_t fb = __float_as_uint(c[j]);
-            return ge_multiple((fb & 0x7FFFFFu) | 0x800000u, (int)(fb >> 23) - 150, m, e) ? m : m - 1u;
-        });
+    for (int j = 0; j < N; ++j) {
+        f[j] = c[j];
+        top = max(top, __float_as_uint(c[j]));
+    }
+    return top > 0x3F800000u;
 }
-
-// FP64 costs: for 2^-126 <= c < 2 the exponent's low 7 bits and the mantissa's
+// FP64: for 2^-126 <= c < 2 the exponent's low 7 bits and the mantissa's
 // leading 23 are those of c truncated to FP32 (relative error below 2^-23), so
 // with the rounding of 1/eps the error is below (floor(1/eps) + 1) * 1.5 *
 // 2^-23, inside e.win.  The high word of a smaller cost is raised to 2^-127's,
@@ -189,8 +179,7 @@ __device__ __forceinline__ void quantise_group(const float (&c)[N], const EpsSpl
 // group the long way: n = 10,000, 1 % ones at eps = 0.3, whole solve 191 ->
 // 241 us.)
 template <int N>
-__device__ __forceinline__ void quantise_group(const double (&c)[N], const EpsSplit &e, uint32_t (&h)[N], bool &bad) {
-    float f[N];
+__device__ __forceinline__ bool group_operands(const double (&c)[N], float (&f)[N]) {
     int top = 0;
     uint32_t signs = 0;
 #pragma unroll
@@ -201,18 +190,38 @@ __device__ __forceinline__ void quantise_group(const double (&c)[N], const EpsSp
         top = max(top, (int)((b - 1ull) >> 32));
         signs |= hi;
     }
+    return top >= 0x3FF00000 || (int)signs < 0;
+}
+
+// One cost the long way; 0 and `bad` for one outside [0, 1].
+__device__ __forceinline__ uint32_t quantise_exact(float c, const EpsSplit &e, bool &bad) {
+    const uint32_t q = quantise_fbits(__float_as_uint(c), e);
+    if (q == 0xFFFFFFFFu) bad = true;
+    return q == 0xFFFFFFFFu ? 0u : q;
+}
+__device__ __forceinline__ uint32_t quantise_exact(double c, const EpsSplit &e, bool &bad) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(c);
+    const uint32_t q = quantise_bits((uint32_t)(b >> 32), (uint32_t)b, e);
+    if (q == 0xFFFFFFFFu) bad = true;
+    return q == 0xFFFFFFFFu ? 0u : q;
+}
+// A cost in [e.low, 1] whose estimate is near the integer m >= 1.
+__device__ __forceinline__ uint32_t quantise_near(float c, uint32_t m, const EpsSplit &e) {
+    const uint32_t b = __float_as_uint(c);
+    return ge_multiple((b & 0x7FFFFFu) | 0x800000u, (int)(b >> 23) - 150, m, e) ? m : m - 1u;
+}
+__device__ __forceinline__ uint32_t quantise_near(double c, uint32_t m, const EpsSplit &e) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(c);
+    return ge_multiple((b & 0xFFFFFFFFFFFFFull) | (1ull << 52), (int)(b >> 52) - 1075, m, e) ? m : m - 1u;
+}
+
+template <int N, class T>
+__device__ __forceinline__ void quantise_group(const T (&c)[N], const EpsSplit &e, uint32_t (&h)[N], bool &bad) {
+    float f[N];
+    const bool out_of_range = group_operands<N>(c, f);
     floor_group<N>(
-        f, e.inv, e.low, e.win, top >= 0x3FF00000 || (int)signs < 0, h,
-        [&](int j) {
-            const unsigned long long b = (unsigned long long)__double_as_longlong(c[j]);
-            const uint32_t q = quantise_bits((uint32_t)(b >> 32), (uint32_t)b, e);
-            if (q == 0xFFFFFFFFu) bad = true;
-            return q == 0xFFFFFFFFu ? 0u : q;
-        },
-        [&](int j, uint32_t m) {
-            const unsigned long long b = (unsigned long long)__double_as_longlong(c[j]);
-            return ge_multiple((b & 0xFFFFFFFFFFFFFull) | (1ull << 52), (int)(b >> 52) - 1075, m, e) ? m : m - 1u;
-        });
+        f, e.inv, e.low, e.win, out_of_range, h, [&](int j) { return quantise_exact(c[j], e, bad); },
+        [&](int j, uint32_t m) { return quantise_near(c[j], m, e); });
 }
 
 // Costs from points: c = RN32(dist / M), dist the squared sum sq or its IEEE
@@ -245,13 +254,22 @@ __device__ __forceinline__ void quantise_points(const float (&sq)[N], int square
         if (!squared) asm("sqrt.approx.f32 %0, %1;" : "=f"(v[j]) : "f"(sq[j]));
         top = max(top, __float_as_uint(sq[j]));
     }
-    const auto exact = [&](int j) {
-        const float d = squared ? sq[j] : __fsqrt_rn(sq[j]);
-        const float c = p.M > 0.0f ? __fdiv_rn(d, p.M) : 0.0f;
-        return exact_cost(d, quantise_fbits(__float_as_uint(c), e));
+    const auto cost = [&](int j, float &d) {
+        d = squared ? sq[j] : __fsqrt_rn(sq[j]);
+        return p.M > 0.0f ? __fdiv_rn(d, p.M) : 0.0f;
     };
-    floor_group<N>(v, p.scale, p.low, 2.0f * e.win, p.wide || top >= 0x7F800000u, h, exact,
-                   [&](int j, uint32_t) { return exact(j); });
+    floor_group<N>(
+        v, p.scale, p.low, 2.0f * e.win, p.wide || top >= 0x7F800000u, h,
+        [&](int j) {
+            float d;
+            const float c = cost(j, d);
+            return exact_cost(d, quantise_fbits(__float_as_uint(c), e));
+        },
+        [&](int j, uint32_t m) {
+            float d;
+            const float c = cost(j, d);
+            return exact_cost(d, quantise_near(c, m, e));
+        });
 }
 
 // Low bytes (16-bit halves) of four values as one stored word (pair).
