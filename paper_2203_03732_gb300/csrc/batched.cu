@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(256, 4) k_bquant_matrix(const T *__restrict__ 
 // kPtRows pairs and the rounded costs are stored 4 (16-bit storage: 8) bytes at
 // a time; the squared sum keeps the operation order of dist_f32.  DIM = 0: any
 // dimension, one pair at a time.  64 clouds of 4096 3-D points (1.07 G pairs):
-// largest distance 0.96 -> 0.35 ms, rounding 2.20 -> 0.68 ms (three loads and about
+// largest distance 0.96 -> 0.35 ms, rounding 2.20 -> 0.63 ms (three loads and about
 // 60 instructions a pair before).
 // ---------------------------------------------------------------------------
 constexpr int kPtRows = 8;

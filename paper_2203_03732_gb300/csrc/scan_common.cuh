@@ -134,13 +134,15 @@ __device__ __forceinline__ uint32_t quantise_fbits(uint32_t fb, const EpsSplit &
 // and exact zeros, common in real costs, stay on the short way.
 // Only the low 8 or 16 bits of h[j] are the result.
 // ---------------------------------------------------------------------------
-template <int N, class Exact, class Settle>
+// ONE (costs from points, where a value takes a square root and a division
+// again): `exact(j)` settles everything, low is not used.
+template <int N, bool ONE, class Exact, class Settle>
 __device__ __forceinline__ void floor_group(const float (&v)[N], float scale, float low, float near, bool out_of_range,
                                             uint32_t (&h)[N], const Exact &exact, const Settle &settle) {
     float d[N], far = 0.0f;
 #pragma unroll
     for (int j = 0; j < N; ++j) {
-        const float x = fmaxf(v[j], low);
+        const float x = ONE ? v[j] : fmaxf(v[j], low);
         const float t = __fmaf_rd(x, scale, 8388608.0f);
         d[j] = __fmaf_rn(x, scale, __fsub_rn(8388607.5f, t));  // 2^23 - 1/2 - t is exact
         far = fmaxf(far, fabsf(d[j]));
@@ -149,8 +151,9 @@ __device__ __forceinline__ void floor_group(const float (&v)[N], float scale, fl
     if (out_of_range || !(far <= 0.5f - near)) {
 #pragma unroll
         for (int j = 0; j < N; ++j) {
-            if (out_of_range) h[j] = exact(j);
-            else if (!(fabsf(d[j]) <= 0.5f - near)) h[j] = settle(j, (h[j] & 0xFFFFu) + (d[j] > 0.0f ? 1u : 0u));
+            const bool close = !(fabsf(d[j]) <= 0.5f - near);
+            if (ONE ? out_of_range || close : out_of_range) h[j] = exact(j);
+            else if (!ONE && close) h[j] = settle(j, (h[j] & 0xFFFFu) + (d[j] > 0.0f ? 1u : 0u));
         }
     }
 }
@@ -219,7 +222,7 @@ template <int N, class T>
 __device__ __forceinline__ void quantise_group(const T (&c)[N], const EpsSplit &e, uint32_t (&h)[N], bool &bad) {
     float f[N];
     const bool out_of_range = group_operands<N>(c, f);
-    floor_group<N>(
+    floor_group<N, false>(
         f, e.inv, e.low, e.win, out_of_range, h, [&](int j) { return quantise_exact(c[j], e, bad); },
         [&](int j, uint32_t m) { return quantise_near(c[j], m, e); });
 }
@@ -232,7 +235,7 @@ __device__ __forceinline__ void quantise_group(const T (&c)[N], const EpsSplit &
 // (all values then, M is the same for all), and NaN.  exact_cost(dist, q) is
 // called with the exact way's distance and result and returns what to store.
 struct PointsScale {
-    float M, scale, low;
+    float M, scale;
     bool wide;
 };
 __device__ __forceinline__ PointsScale points_scale(uint32_t max_sq_bits, int squared, const EpsSplit &e) {
@@ -240,7 +243,6 @@ __device__ __forceinline__ PointsScale points_scale(uint32_t max_sq_bits, int sq
     p.M = squared ? __uint_as_float(max_sq_bits) : __fsqrt_rn(__uint_as_float(max_sq_bits));
     p.wide = !(p.M >= 1e-18f && p.M <= 1e18f);
     p.scale = p.wide ? 0.0f : __fdiv_rn(e.inv, p.M);
-    p.low = __fmul_rn(e.low, p.M);
     return p;
 }
 template <int N, class Cost>
@@ -254,22 +256,14 @@ __device__ __forceinline__ void quantise_points(const float (&sq)[N], int square
         if (!squared) asm("sqrt.approx.f32 %0, %1;" : "=f"(v[j]) : "f"(sq[j]));
         top = max(top, __float_as_uint(sq[j]));
     }
-    const auto cost = [&](int j, float &d) {
-        d = squared ? sq[j] : __fsqrt_rn(sq[j]);
-        return p.M > 0.0f ? __fdiv_rn(d, p.M) : 0.0f;
-    };
-    floor_group<N>(
-        v, p.scale, p.low, 2.0f * e.win, p.wide || top >= 0x7F800000u, h,
+    floor_group<N, true>(
+        v, p.scale, 0.0f, 2.0f * e.win, p.wide || top >= 0x7F800000u, h,
         [&](int j) {
-            float d;
-            const float c = cost(j, d);
+            const float d = squared ? sq[j] : __fsqrt_rn(sq[j]);
+            const float c = p.M > 0.0f ? __fdiv_rn(d, p.M) : 0.0f;
             return exact_cost(d, quantise_fbits(__float_as_uint(c), e));
         },
-        [&](int j, uint32_t m) {
-            float d;
-            const float c = cost(j, d);
-            return exact_cost(d, quantise_near(c, m, e));
-        });
+        [](int, uint32_t) { return 0u; });
 }
 
 // Low bytes (16-bit halves) of four values as one stored word (pair).
