@@ -15,7 +15,9 @@ torch-facing wrapper (device memory, streams, argument marshalling).
 """
 from __future__ import annotations
 
+import collections
 import ctypes
+import threading
 
 from . import _lib
 
@@ -32,29 +34,73 @@ def _torch():
 
 
 class Workspace:
-    """A reusable device workspace (grown on demand, 256-byte aligned)."""
+    """A reusable device workspace (grown on demand, 256-byte aligned).  It
+    serves one solve at a time: solves that may overlap (on several streams,
+    or enqueued by several threads) need one each."""
 
     def __init__(self, device=None):
         torch = _torch()
         self.device = torch.device(device if device is not None else "cuda")
         self.buf = None
+        self.stream = None  # the stream of the last solve
+        self._streams = set()
 
     def get(self, nbytes: int):
         torch = _torch()
+        self.stream = torch.cuda.current_stream(self.device)
         if self.buf is None or self.buf.numel() < nbytes:
             self.buf = torch.empty(max(nbytes, 256), dtype=torch.uint8, device=self.device)
+            self._streams = {self.stream.cuda_stream}
+        elif self.stream.cuda_stream not in self._streams:
+            # a buffer that is outgrown or dropped is not given to another
+            # tensor before the work of every stream that used it
+            self.buf.record_stream(self.stream)
+            self._streams.add(self.stream.cuda_stream)
         assert self.buf.data_ptr() % 256 == 0
         return self.buf
 
 
-_default_ws = {}
+# The workspaces of calls without `ws`: one per thread and stream, so that
+# asynchronous calls on several streams or from several threads share none.  A
+# thread keeps those of the streams it used last; a buffer goes back to the
+# allocator in the order of the stream it was allocated and used on.
+_DEFAULT_WS_PER_THREAD = 8
+_default_ws = threading.local()
+_last_default_ws = {}  # by device, for ws_status
+
+
+def _device_index(torch, device):
+    return device.index if device.index is not None else torch.cuda.current_device()
 
 
 def _workspace(device):
-    key = str(device)
-    if key not in _default_ws:
-        _default_ws[key] = Workspace(device)
-    return _default_ws[key]
+    torch = _torch()
+    device = torch.device(device)
+    dev = _device_index(torch, device)
+    if torch.cuda.is_current_stream_capturing():
+        ws = Workspace(device)  # a graph's buffers are its own
+    else:
+        cache = _default_ws.__dict__.setdefault("by_stream", collections.OrderedDict())
+        key = (dev, torch.cuda.current_stream(device).cuda_stream)
+        ws = cache.get(key)
+        if ws is None:
+            ws = cache[key] = Workspace(device)
+            if len(cache) > _DEFAULT_WS_PER_THREAD:
+                cache.popitem(last=False)
+        else:
+            cache.move_to_end(key)
+    _default_ws.__dict__.setdefault("last", {})[dev] = _last_default_ws[dev] = ws
+    return ws
+
+
+def _status_workspace(torch):
+    """The default workspace that ws_status reads: the calling thread's for the
+    current stream, else its last on the current device, else any thread's."""
+    dev = torch.cuda.current_device()
+    here = _default_ws.__dict__
+    key = (dev, torch.cuda.current_stream().cuda_stream)
+    return (here.get("by_stream", {}).get(key) or here.get("last", {}).get(dev) or _last_default_ws.get(dev)
+            or Workspace(torch.device("cuda", dev)))
 
 
 def _stream_handle(torch, device):
@@ -62,13 +108,18 @@ def _stream_handle(torch, device):
 
 
 def ws_status(ws: Workspace | None = None):
-    """Raise PrError if a solve enqueued on `ws` (default: the current
-    device's default workspace) recorded a device-side error; synchronises
-    the current stream (pr_ws_status).  For calls made with sync=False."""
+    """Raise PrError if the last solve enqueued on `ws` recorded a device-side
+    error; waits for it and synchronises the current stream (pr_ws_status).
+    For calls made with sync=False.  Default: the workspace of this thread's
+    calls without `ws` on the current stream (else its last on the current
+    device, else any thread's)."""
     torch = _torch()
-    w = ws or _workspace(torch.device("cuda", torch.cuda.current_device()))
+    w = ws or _status_workspace(torch)
     if w.buf is None:
         raise ValueError("ws_status: the workspace holds no solve")
+    cur = torch.cuda.current_stream(w.buf.device)
+    if w.stream is not None and w.stream != cur:
+        cur.wait_stream(w.stream)
     _lib.check(_lib.load().pr_ws_status(w.buf.data_ptr(), _stream_handle(torch, w.buf.device)), "pr_ws_status")
 
 
