@@ -1885,13 +1885,18 @@ int max_phase_cluster(size_t smem) {
 
 
 
+// The launch limits of the current device, found on its first call; calls come
+// from any thread.
 pr_status phase_cfg(PhaseCfg &cfg) {
-    static int cached_dev = -1;
-    static PhaseCfg cached;
+    constexpr int kMaxDevices = 64;
+    static std::mutex mu;
+    static PhaseCfg cached[kMaxDevices];  // grid 0: not found yet
     int dev = 0;
     PR_CUDA(cudaGetDevice(&dev));
-    if (dev == cached_dev) {
-        cfg = cached;
+    if (dev < 0 || dev >= kMaxDevices) return fail(PR_ERR_INVALID, "device %d: need 0 <= device < %d", dev, kMaxDevices);
+    std::lock_guard<std::mutex> lock(mu);
+    if (cached[dev].grid > 0) {
+        cfg = cached[dev];
         return PR_OK;
     }
     const DeviceInfo &di = device_info();
@@ -1916,6 +1921,8 @@ pr_status phase_cfg(PhaseCfg &cfg) {
     if (rc == PR_OK) rc = set_phase_attrs<uint8_t, false, true, true, true>(smem);
     if (rc == PR_OK) rc = set_phase_attrs<uint8_t, true, true, true, true>(smem);
     if (rc != PR_OK) return rc;
+    PR_CUDA(cudaFuncSetAttribute(k_seq<uint8_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSeqMaxKeyBytes));
+    PR_CUDA(cudaFuncSetAttribute(k_seq<uint16_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSeqMaxKeyBytes));
     int per_sm = 0, per_sm16 = 0;
     PR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_phases<uint8_t, false, false, false, false>, kThreads, smem));
     PR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm16, k_phases<uint16_t, false, false, false, false>, kThreads, smem));
@@ -1927,8 +1934,7 @@ pr_status phase_cfg(PhaseCfg &cfg) {
     const int c8 = max_phase_cluster<uint8_t>(smem), c16 = max_phase_cluster<uint16_t>(smem);
     cfg.cluster = c8 < c16 ? c8 : c16;
     cfg.smem = smem;  // the most a launch may ask for; each launch asks smem_bytes(ldq)
-    cached = cfg;
-    cached_dev = dev;
+    cached[dev] = cfg;
     return PR_OK;
 }
 
@@ -2159,7 +2165,6 @@ pr_status launch_solve(Params &p, const CostSource &src, double eps, const Phase
         // was checked by pr_assign_rule)
         const size_t ksm = (size_t)p.ldq * (cb8 ? 1 : 2);
         const void *fn = cb8 ? (const void *)k_seq<uint8_t> : (const void *)k_seq<uint16_t>;
-        PR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ksm));
         Params pc = p;
         void *args[] = {(void *)&pc};
         PR_CUDA(cudaLaunchCooperativeKernel(fn, dim3(cfg.grid), dim3(kThreads), args, ksm, st));
