@@ -350,6 +350,23 @@ def _autotune(torch, L, dev, kind, args_src, sizes, n_ptr, eps, out, wsb):
     return (best.threads, best.ctas_per_sm)
 
 
+def _tuned(torch, L, dev, kind, extra, args_src, n, n_ptr, eps, out, wsb):
+    """The remembered launch shape for this batch, else the autotuner's, which
+    is then remembered.  None (the default shape) where the batch has invalid
+    costs: the solve itself reports them."""
+    key = _tune_key(torch, dev, kind, n, eps, extra=extra)
+    tune = _tune_lookup(key)
+    if tune is None:
+        try:
+            tune = _autotune(torch, L, dev, kind, args_src, n, n_ptr, eps, out, wsb)
+        except PrError as e:
+            if e.status != _lib.PR_ERR_INVALID:
+                raise
+            return None
+        _tune_store(key, tune)
+    return tune
+
+
 def _tune_struct(tune):
     if tune is None:
         return None
@@ -406,12 +423,8 @@ def assign_batched(C, sizes, eps: float, *, tune=None, sync: bool = True,
     wsb = (ws or _workspace(dev)).get(need)
     out = out or _batched_outputs(torch, dev, n)
     if isinstance(tune, str):
-        key = _tune_key(torch, dev, "matrix", n, eps, extra=str(C.dtype))
-        tune = _tune_lookup(key)
-        if tune is None:
-            tune = _autotune(torch, L, dev, "matrix", (None, None, 0, 0, C.data_ptr(), dt), n, n_ptr, eps,
-                             out, wsb)
-            _tune_store(key, tune)
+        tune = _tuned(torch, L, dev, "matrix", str(C.dtype), (None, None, 0, 0, C.data_ptr(), dt), n, n_ptr, eps,
+                      out, wsb)
     st = _lib.PrStats()
     rc = L.pr_assign_batched(C.data_ptr(), dt, len(n), n_ptr, float(eps),
                              out["row_to_col"].data_ptr(), out["col_to_row"].data_ptr(),
@@ -455,12 +468,8 @@ def assign_batched_points(XA, XB, sizes, eps: float, *, metric: str = "sqeuclide
     wsb = (ws or _workspace(dev)).get(need)
     out = out or _batched_outputs(torch, dev, n)
     if isinstance(tune, str):
-        key = _tune_key(torch, dev, "points", n, eps, extra=f"{metric}d{XA.shape[1]}")
-        tune = _tune_lookup(key)
-        if tune is None:
-            tune = _autotune(torch, L, dev, "points", (XA.data_ptr(), XB.data_ptr(), XA.shape[1], m, None, 0),
-                             n, n_ptr, eps, out, wsb)
-            _tune_store(key, tune)
+        tune = _tuned(torch, L, dev, "points", f"{metric}d{XA.shape[1]}",
+                      (XA.data_ptr(), XB.data_ptr(), XA.shape[1], m, None, 0), n, n_ptr, eps, out, wsb)
     st = _lib.PrStats()
     rc = L.pr_assign_batched_points(XA.data_ptr(), XB.data_ptr(), XA.shape[1], m, len(n), n_ptr,
                                     float(eps), out["row_to_col"].data_ptr(),

@@ -737,8 +737,11 @@ extern "C" pr_status pr_assign_batched_autotune(const float *XA, const float *XB
     cudaEventDestroy(e1);
     if (best_t < 0.0f) return fail(last_err != PR_OK ? last_err : PR_ERR_INVALID,
                                    "pr_assign_batched_autotune: no launch shape worked");
-    // the solve with the chosen shape leaves its results in the outputs
-    const pr_status rc = run(&bt);
+    // the solve with the chosen shape leaves its results in the outputs; an error
+    // found on the device (costs out of range) stops every candidate's solve, so
+    // the times tell nothing
+    pr_status rc = run(&bt);
+    if (rc == PR_OK) rc = pr_ws_status(ws, stream);
     if (rc != PR_OK) return rc;
     *best = bt;
     *best_ms = best_t;
