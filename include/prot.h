@@ -236,7 +236,8 @@ pr_status pr_dual_bound(const int32_t *y_row, const int32_t *y_col, int32_t n_ro
 
 /* Launch shape of the batched solver (0 = default). */
 typedef struct {
-    int32_t threads;     /* threads per solver CTA: 128, 256, 512 or 1024 (0 = by the largest problem) */
+    int32_t threads;     /* threads per solver CTA: 128, 256, 512 or 1024 (0 = by the largest
+                            problem, the number of problems and eps) */
     int32_t ctas_per_sm; /* resident solver CTAs per SM, 0 = as many as fit        */
 } pr_batched_tune;
 

@@ -1608,6 +1608,7 @@ struct SoloCost {
 // RESUME: the first phases ran in k_phases (SEQ: k_seq), which stopped at a
 // few free rows or inside a phase: the state is taken over from its words,
 // keys, duals and row lists.
+// SEQ (always with RESUME): the sequential rule.
 template <class CB, bool F7, bool RESUME, bool SEQ>
 __global__ void __launch_bounds__(kSoloThreads)
 k_solo(Params p, SoloCost src, int *match_b, int *match_a, int *y_col, double *cost) {
@@ -1669,7 +1670,7 @@ k_solo(Params p, SoloCost src, int *match_b, int *match_a, int *y_col, double *c
     }
     __syncthreads();
     const CB *cb = static_cast<const CB *>(p.cb);
-    if (SEQ) cta_seq_phases<4, CB, F7>(s, st, cb, p.nA, p.ldq, p.T, p.phase_cap, RESUME ? 1u : 0u, nf, c);
+    if (SEQ) cta_seq_phases<4, CB, F7>(s, st, cb, p.nA, p.ldq, p.T, p.phase_cap, 1u, nf, c);
     else cta_phases<4, CB, F7, true>(s, st, cb, p.nB, p.nA, p.ldq, p.T, p.phase_cap, RESUME ? 1u : 0u, nf, mid, c);
     if (threadIdx.x == 0) {
         ctl->phases = c.phases;
@@ -1942,7 +1943,8 @@ pr_status phase_cfg(PhaseCfg &cfg) {
 // distributed shared memory, about a third of a grid barrier's latency), on
 // the whole grid (one CTA per SM, barriers through L2), on one CTA, or on the
 // grid and then on one CTA.  PR_PHASE_MODE = "grid", "cluster", "solo" or
-// "hand" forces one (the last two where they fit).
+// "hand" forces one (the last two where they fit; the sequential rule knows
+// "grid" and, for any other, "hand").
 // Cluster mode also needs at least kMinSlots row slots next to the keys.
 constexpr int kMinSlots = 4;
 
@@ -1950,9 +1952,9 @@ constexpr int kMinSlots = 4;
 // rows at floor(1/eps) > 20 (its two jobs per row keep 16 SMs busy; at larger
 // eps a solve is one phase of many rounds with many rows, where the whole
 // grid's scans win).  The lowest-index rule takes one CTA for its small rounds
-// instead (use_cta), and where it does not the grid is ahead (ms, cluster /
-// grid: n = 3000, eps = 0.02 0.714 / 0.655; n = 4000, eps = 0.02 0.832 /
-// 0.730, eps = 0.01 2.94 / 2.79).
+// instead (use_cta), and where it does not the grid is ahead (us, cluster /
+// grid: 300 x 8000, eps = 0.02 46 / 42; 300 x 16,000 50 / 47; n = 3000 714 / 655;
+// n = 4000 832 / 730, 0.01 2940 / 2790): for it the cluster runs only when forced.
 constexpr int kClusterMaxRows = 4096;
 constexpr long long kClusterMinK = 20;
 
@@ -2217,8 +2219,7 @@ pr_status launch_solve(Params &p, const CostSource &src, double eps, const Phase
         const SoloCost cost_src{src.points ? nullptr : C, ldc, dt == PR_F64,
                                 PointsCost{src.XA, src.XB, src.dim, src.squared}};
         const bool seq = p.rule == PR_RULE_SEQUENTIAL;
-        const auto launch = solo ? (seq ? launch_solo<false, true> : launch_solo<false, false>)
-                                 : (seq ? launch_solo<true, true> : launch_solo<true, false>);
+        const auto launch = solo ? launch_solo<false, false> : seq ? launch_solo<true, true> : launch_solo<true, false>;
         const pr_status rc = launch(p, cost_src, cb8, f7, row_to_col, col_to_row, y_col, cost, st);
         if (rc != PR_OK) return rc;
     }
@@ -2470,7 +2471,7 @@ constexpr size_t kNoAllocBytes = (size_t)2304 * 1024;
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
 
 struct NoAllocLayout {
-    size_t ctl, cb, ka, prop, won, pool, part, lists, total;
+    size_t ctl, cb, ka, prop, won, pool, lists, total;
     int ldq, won_words;
 };
 
@@ -2487,7 +2488,6 @@ NoAllocLayout make_noalloc_layout(int nB, int nA) {
     L.won_words = (nA + 31) / 32;
     L.won = c.take<unsigned>(3 * (size_t)L.won_words);
     L.pool = c.take<int2>(2 * (size_t)nB);
-    L.part = c.take<double>(1024);
     L.lists = c.take<int>(2 * (size_t)nB);  // completion scratch
     L.total = c.total();
     return L;
@@ -2548,7 +2548,6 @@ extern "C" pr_status pr_assign_noalloc(const void *C, pr_dtype dt, int64_t ldc, 
     p.won = (unsigned *)(w + L.won);
     p.won_words = L.won_words;
     p.pool = (int2 *)(w + L.pool);
-    p.part = (double *)(w + L.part);
     p.lists = (int *)(w + L.lists);
     p.list_stride = 0;  // no overflow region: never addressed for n_rows <= 1024
     p.nB = n_rows;

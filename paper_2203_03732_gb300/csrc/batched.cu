@@ -75,7 +75,6 @@ struct BParams {
     BCtl *ctl;
     const BDesc *desc;
     const int *order;
-    const unsigned *maxbits;
     const void *cb;  // uint8_t or uint16_t, as k_bsolve is instantiated
     int nprob;
     int n_max;
@@ -580,7 +579,6 @@ pr_status run_batched(const Source &src, int32_t P, const int32_t *n_host, doubl
     bp.ctl = ctl;
     bp.desc = d_desc;
     bp.order = d_order;
-    bp.maxbits = d_max;
     bp.cb = d_cb;
     bp.nprob = P;
     bp.n_max = pl.n_max;

@@ -79,7 +79,7 @@ inline CtaChoice choose_cta(bool seq, int n_rows, int n_cols, int row_bytes, int
                             const char *mode) {
     CtaChoice c;
     if (mode && (strcmp(mode, "grid") == 0 || strcmp(mode, "cluster") == 0)) return c;
-    if (mode ? strcmp(mode, "solo") == 0 : !seq && solo_fits(n_rows, n_cols, row_bytes, K)) {
+    if (!seq && (mode ? strcmp(mode, "solo") == 0 : solo_fits(n_rows, n_cols, row_bytes, K))) {
         c.solo = true;
         return c;
     }

@@ -44,6 +44,7 @@ def test_rows_kept_by_the_grids_ctas_are_never_taken_over(choose):
     assert choose(1500, 1500, 0.1, ctas=6)["mid"]
     assert choose(1500, 1500, 0.1, ctas=5) == dict(solo=False, hand=0, mid=False)
     assert choose(6000, 6000, 0.005, ctas=20, mode=b"hand")["hand"] == 0
+    assert choose(300, 300, 0.01, seq=True, mode=b"solo") == dict(solo=False, hand=64, mid=False)
     # the sequential rule's ring holds every row
     assert choose(6000, 6000, 0.003, ctas=20, seq=True)["hand"] == choose(6000, 6000, 0.003, seq=True)["hand"]
 
