@@ -33,6 +33,12 @@ def _torch():
     return torch
 
 
+def _raw_stream(torch, index):
+    """The current stream's handle on a device (the torch.cuda.Stream object
+    takes 2 us to make, which counts in the smallest calls)."""
+    return torch._C._cuda_getCurrentRawStream(index)
+
+
 class Workspace:
     """A reusable device workspace (grown on demand, 256-byte aligned).  It
     serves one solve at a time: solves that may overlap (on several streams,
@@ -42,21 +48,25 @@ class Workspace:
         torch = _torch()
         self.device = torch.device(device if device is not None else "cuda")
         self.buf = None
-        self.stream = None  # the stream of the last solve
+        self.stream = None  # handle of the last solve's stream
         self._streams = set()
+        self._index = self.device.index
 
     def get(self, nbytes: int):
         torch = _torch()
-        self.stream = torch.cuda.current_stream(self.device)
         if self.buf is None or self.buf.numel() < nbytes:
             self.buf = torch.empty(max(nbytes, 256), dtype=torch.uint8, device=self.device)
-            self._streams = {self.stream.cuda_stream}
-        elif self.stream.cuda_stream not in self._streams:
+            self._index = self.buf.device.index
+            self.stream = _raw_stream(torch, self._index)
+            self._streams = {self.stream}
+            assert self.buf.data_ptr() % 256 == 0
+            return self.buf
+        self.stream = _raw_stream(torch, self._index)
+        if self.stream not in self._streams:
             # a buffer that is outgrown or dropped is not given to another
             # tensor before the work of every stream that used it
-            self.buf.record_stream(self.stream)
-            self._streams.add(self.stream.cuda_stream)
-        assert self.buf.data_ptr() % 256 == 0
+            self.buf.record_stream(torch.cuda.current_stream(self._index))
+            self._streams.add(self.stream)
         return self.buf
 
 
@@ -66,30 +76,28 @@ class Workspace:
 # allocator in the order of the stream it was allocated and used on.
 _DEFAULT_WS_PER_THREAD = 8
 _default_ws = threading.local()
-_last_default_ws = {}  # by device, for ws_status
-
-
-def _device_index(torch, device):
-    return device.index if device.index is not None else torch.cuda.current_device()
+_last_default_ws = {}  # by device index, for ws_status
 
 
 def _workspace(device):
     torch = _torch()
-    device = torch.device(device)
-    dev = _device_index(torch, device)
+    dev = device.index if device.index is not None else torch.cuda.current_device()
+    here = _default_ws.__dict__
     if torch.cuda.is_current_stream_capturing():
-        ws = Workspace(device)  # a graph's buffers are its own
+        ws = Workspace(torch.device("cuda", dev))  # a graph's buffers are its own
     else:
-        cache = _default_ws.__dict__.setdefault("by_stream", collections.OrderedDict())
-        key = (dev, torch.cuda.current_stream(device).cuda_stream)
+        cache = here.get("by_stream")
+        if cache is None:
+            cache = here["by_stream"] = collections.OrderedDict()
+        key = (dev, _raw_stream(torch, dev))
         ws = cache.get(key)
         if ws is None:
-            ws = cache[key] = Workspace(device)
+            ws = cache[key] = Workspace(torch.device("cuda", dev))
             if len(cache) > _DEFAULT_WS_PER_THREAD:
                 cache.popitem(last=False)
         else:
             cache.move_to_end(key)
-    _default_ws.__dict__.setdefault("last", {})[dev] = _last_default_ws[dev] = ws
+    here.setdefault("last", {})[dev] = _last_default_ws[dev] = ws
     return ws
 
 
@@ -98,13 +106,13 @@ def _status_workspace(torch):
     current stream, else its last on the current device, else any thread's."""
     dev = torch.cuda.current_device()
     here = _default_ws.__dict__
-    key = (dev, torch.cuda.current_stream().cuda_stream)
-    return (here.get("by_stream", {}).get(key) or here.get("last", {}).get(dev) or _last_default_ws.get(dev)
-            or Workspace(torch.device("cuda", dev)))
+    return (here.get("by_stream", {}).get((dev, _raw_stream(torch, dev))) or here.get("last", {}).get(dev)
+            or _last_default_ws.get(dev) or Workspace(torch.device("cuda", dev)))
 
 
 def _stream_handle(torch, device):
-    return ctypes.c_void_p(torch.cuda.current_stream(device).cuda_stream)
+    return ctypes.c_void_p(_raw_stream(torch, device.index if device.index is not None
+                                       else torch.cuda.current_device()))
 
 
 def ws_status(ws: Workspace | None = None):
@@ -117,10 +125,11 @@ def ws_status(ws: Workspace | None = None):
     w = ws or _status_workspace(torch)
     if w.buf is None:
         raise ValueError("ws_status: the workspace holds no solve")
-    cur = torch.cuda.current_stream(w.buf.device)
-    if w.stream is not None and w.stream != cur:
-        cur.wait_stream(w.stream)
-    _lib.check(_lib.load().pr_ws_status(w.buf.data_ptr(), _stream_handle(torch, w.buf.device)), "pr_ws_status")
+    dev = w.buf.device
+    if w.stream is not None and w.stream != _raw_stream(torch, dev.index):
+        used = torch.cuda.ExternalStream(w.stream, dev) if w.stream else torch.cuda.default_stream(dev)
+        torch.cuda.current_stream(dev).wait_stream(used)
+    _lib.check(_lib.load().pr_ws_status(w.buf.data_ptr(), _stream_handle(torch, dev)), "pr_ws_status")
 
 
 def assign(C, eps: float, *, sync: bool = True, ws: Workspace | None = None, out=None,

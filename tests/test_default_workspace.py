@@ -17,16 +17,16 @@ import paper_2203_03732_gb300 as prot
 @pytest.fixture
 def streams(monkeypatch):
     """set(handle) makes `handle` the current stream of the device."""
-    cur = types.SimpleNamespace(cuda_stream=0)
+    cur = types.SimpleNamespace(handle=0)
     cap = types.SimpleNamespace(on=False)
-    monkeypatch.setattr(torch.cuda, "current_stream", lambda *a: types.SimpleNamespace(cuda_stream=cur.cuda_stream))
+    monkeypatch.setattr(prot, "_raw_stream", lambda *a: cur.handle)
     monkeypatch.setattr(torch.cuda, "current_device", lambda: 0)
     monkeypatch.setattr(torch.cuda, "is_current_stream_capturing", lambda: cap.on)
     monkeypatch.setattr(prot, "_default_ws", threading.local())
     monkeypatch.setattr(prot, "_last_default_ws", {})
 
     def set_(handle, capturing=False):
-        cur.cuda_stream, cap.on = handle, capturing
+        cur.handle, cap.on = handle, capturing
     return set_
 
 
