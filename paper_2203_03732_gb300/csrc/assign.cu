@@ -2041,11 +2041,8 @@ StageRes g_stage[kStageMaxDevices];
 template <class T, class CB>
 void launch_quantise_rows(const CostSource &src, const Params &p, int r0, int rows, double eps, int sms,
                           cudaStream_t st) {
-    const long long groups = (long long)rows * (p.ldq >> 3);
-    const long long want = groups / 256 + 1;
-    const int grid = (int)(want < (long long)sms * 16 ? want : (long long)sms * 16);
     launch_quantise<T, CB>((const T *)src.C + (size_t)r0 * src.ldc, src.ldc, rows, p.nA, p.ldq, eps,
-                           (CB *)const_cast<void *>(p.cb) + (size_t)r0 * p.ldq, &p.ctl->head, grid, st);
+                           (CB *)const_cast<void *>(p.cb) + (size_t)r0 * p.ldq, &p.ctl->head, sms, st);
 }
 
 // Eq. 1 for a host matrix: its rows go to the device buffer src.C in chunks
@@ -2121,9 +2118,6 @@ pr_status launch_solve(Params &p, const CostSource &src, double eps, const Phase
     if (solo) k_solo_init<<<1, 256, 0, st>>>(p.ctl);
     else k_init<<<di.sms * 2, 256, 0, st>>>(p, row_to_col);
     PR_CUDA(cudaGetLastError());
-    const long long groups = (long long)n_rows * (p.ldq >> 3);
-    const long long want = groups / 256 + 1;
-    const int qgrid = (int)(want < (long long)di.sms * 16 ? want : (long long)di.sms * 16);
     void *cbw = const_cast<void *>(p.cb);
     if (src.points) {
         const EpsSplit e = make_eps_split(eps);
@@ -2135,16 +2129,16 @@ pr_status launch_solve(Params &p, const CostSource &src, double eps, const Phase
         if (rc != PR_OK) return rc;
     } else if (dt == PR_F64 && cb8)
         launch_quantise<double, uint8_t>((const double *)C, ldc, n_rows, n_cols, p.ldq, eps, (uint8_t *)cbw,
-                                         &p.ctl->head, qgrid, st);
+                                         &p.ctl->head, di.sms, st);
     else if (dt == PR_F64)
         launch_quantise<double, uint16_t>((const double *)C, ldc, n_rows, n_cols, p.ldq, eps, (uint16_t *)cbw,
-                                          &p.ctl->head, qgrid, st);
+                                          &p.ctl->head, di.sms, st);
     else if (cb8)
         launch_quantise<float, uint8_t>((const float *)C, ldc, n_rows, n_cols, p.ldq, eps, (uint8_t *)cbw,
-                                        &p.ctl->head, qgrid, st);
+                                        &p.ctl->head, di.sms, st);
     else
         launch_quantise<float, uint16_t>((const float *)C, ldc, n_rows, n_cols, p.ldq, eps, (uint16_t *)cbw,
-                                         &p.ctl->head, qgrid, st);
+                                         &p.ctl->head, di.sms, st);
     PR_CUDA(cudaGetLastError());
 
     const int chunk = cb8 ? kChunk<uint8_t> : kChunk<uint16_t>;

@@ -1160,22 +1160,19 @@ extern "C" pr_status pr_ot(const void *C, pr_dtype dt, int64_t ldc, int32_t n_su
     else k_ot_init<uint16_t><<<g1 * 4, 256, 0, st>>>(p);
     PR_CUDA(cudaGetLastError());
     {
-        const long long groups = (long long)nB * (L.ldq >> 3);
-        const long long want = groups / 256 + 1;
-        const int qgrid = (int)std::min<long long>(want, (long long)di.sms * 16);
         void *cbw = const_cast<void *>(p.cb);
         if (dt == PR_F64 && cb8)
             launch_quantise<double, uint8_t>((const double *)C, ldc, nB, nA, L.ldq, eps, (uint8_t *)cbw,
-                                             &p.ctl->head, qgrid, st);
+                                             &p.ctl->head, di.sms, st);
         else if (dt == PR_F64)
             launch_quantise<double, uint16_t>((const double *)C, ldc, nB, nA, L.ldq, eps, (uint16_t *)cbw,
-                                              &p.ctl->head, qgrid, st);
+                                              &p.ctl->head, di.sms, st);
         else if (cb8)
             launch_quantise<float, uint8_t>((const float *)C, ldc, nB, nA, L.ldq, eps, (uint8_t *)cbw,
-                                            &p.ctl->head, qgrid, st);
+                                            &p.ctl->head, di.sms, st);
         else
             launch_quantise<float, uint16_t>((const float *)C, ldc, nB, nA, L.ldq, eps, (uint16_t *)cbw,
-                                             &p.ctl->head, qgrid, st);
+                                             &p.ctl->head, di.sms, st);
         PR_CUDA(cudaGetLastError());
     }
     const int gw = di.sms * 8;  // warps-per-row kernels of the fix-up: grid of 256-thread CTAs

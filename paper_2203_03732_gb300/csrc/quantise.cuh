@@ -66,14 +66,19 @@ __device__ __forceinline__ void round_chunk(const T *__restrict__ row, int n, in
 // ---------------------------------------------------------------------------
 // k_quantise: Eq. (1) exactly.  With VEC (rows 16-byte aligned) a thread takes
 // 8 columns with 16-byte loads; otherwise a warp takes a chunk of a row.
-// Bound by HBM: n = 10,000 FP64 to bytes (0.9 GB) 147 -> 130 us (6.9 TB/s),
-// FP32 (0.5 GB) 90 -> 82 us, 2999 x 4507 FP32 (unaligned) 18 -> 13.5 us with
-// quantise_group.
+// Bound by HBM: n = 10,000 FP64 to bytes (0.9 GB) 129 us (7.0 TB/s; 147 one cost
+// at a time), FP32 (0.5 GB) 77 us (92), 9999 x 9999 (rows off 16 bytes) FP64 137
+// us (194), FP32 77 us (105).
 // ---------------------------------------------------------------------------
+// CTAs per SM of the grid.  With VEC those that are resident at once, 5 (the
+// launch bound holds the registers to 48): n = 10,000 FP64 131 us, FP32 77 us;
+// 16 per SM, a last wave of one fifth, 136 and 83 us.  The other form, 6
+// resident, runs four waves (n = 9999 FP64 137 us; one wave 139, 5 per SM 156).
+constexpr int kRoundCtas = 5, kRoundCtasUnaligned = 24;
 // CB is the stored type: uint16_t, or uint8_t when every cbar <= 252 (the
 // caller checks floor(1/eps) <= 252); padding columns get 0x7FFF / 0xFF.
 template <class T, bool VEC, class CB>
-__global__ void k_quantise(const T *__restrict__ C, long long ldc, int nB, int nA, int ldq,
+__global__ void __launch_bounds__(256, VEC ? 5 : 6) k_quantise(const T *__restrict__ C, long long ldc, int nB, int nA, int ldq,
                            EpsSplit e, CB *__restrict__ cb, WsHead *head) {
     constexpr uint32_t kPad = sizeof(CB) == 1 ? 0xFFu : (uint32_t)kPadCost;
     bool bad = false;
@@ -145,9 +150,11 @@ __global__ void k_quantise(const T *__restrict__ C, long long ldc, int nB, int n
 // Launch k_quantise with 16-byte loads when every row starts 16-byte aligned.
 template <class T, class CB = uint16_t>
 void launch_quantise(const T *C, long long ldc, int nB, int nA, int ldq, double eps, CB *cb,
-                     WsHead *head, int grid, cudaStream_t st) {
+                     WsHead *head, int sms, cudaStream_t st) {
     const EpsSplit e = make_eps_split(eps);
     const bool vec = ((uintptr_t)C % 16 == 0) && ((ldc * (long long)sizeof(T)) % 16 == 0);
+    const long long want = (long long)nB * (ldq >> 3) / 256 + 1, most = (long long)sms * (vec ? kRoundCtas : kRoundCtasUnaligned);
+    const int grid = (int)(want < most ? want : most);
     if (vec) k_quantise<T, true, CB><<<grid, 256, 0, st>>>(C, ldc, nB, nA, ldq, e, cb, head);
     else k_quantise<T, false, CB><<<grid, 256, 0, st>>>(C, ldc, nB, nA, ldq, e, cb, head);
 }
