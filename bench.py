@@ -165,7 +165,8 @@ class ClockSampler:
 
 # The sources the phase kernel is built from (its translation unit and the
 # headers it includes): the captured DRAM traffic stays valid while they do.
-PHASE_SOURCES = ("assign.cu", "scan_common.cuh", "quantise.cuh", "points.cuh", "prot_internal.cuh")
+PHASE_SOURCES = ("assign.cu", "scan_common.cuh", "quantise.cuh", "points.cuh", "prot_internal.cuh", "cta_solve.cuh",
+                 "cta_choice.cuh", "rule_ii.cuh", "rule_seq.cuh")
 
 
 def src_hash():

@@ -99,7 +99,9 @@ struct Ctl {
     // prof_own sums CTA 0's values over the rounds, prof_max sums the
     // per-round maximum over CTAs of each segment; prof_rounds counts rounds.
     // The sequential rule (rule_seq.cuh) uses them per phase: segments key
-    // update, chains, both; prof_own[3] sums the warps per row.
+    // update, chains, both; prof_own[3] sums the warps per row.  A profiled
+    // solve runs on the grid alone, without fast rounds and take-overs: the
+    // split is of the rounds with many rows.
     unsigned long long prof_own[8];
     unsigned long long prof_max[8];
     unsigned long long prof_slot[2][8];  // per round parity: max over CTAs

@@ -319,7 +319,7 @@ __device__ void write_unsolved(const BParams &p, const BDesc &D, int pi) {
 // CTAs per SM the registers are held to: 128 registers a thread at 128 and 256
 // threads, so that 4 and 2 CTAs fit (the compiler takes 172 otherwise, and one
 // CTA of 256 threads sat alone on an SM: 512 problems of up to 2048 rows 2.69
-// -> 2.00 ms).  85 and 64 registers spill: that batch 1.90 and 1.86 ms, but 300
+// -> 2.00 ms, 1.93 now).  85 and 64 registers spill: that batch 1.90 and 1.86 ms, but 300
 // problems of up to 700 rows 0.73 -> 0.85 and 0.91 ms.
 template <int THREADS>
 constexpr int kSolveCtas = THREADS == 128 ? 4 : THREADS == 256 ? 2 : 1;
@@ -459,10 +459,10 @@ pr_status run_batched(const Source &src, int32_t P, const int32_t *n_host, doubl
     // Threads per CTA by the largest problem: short rows and few of them want
     // cheap CTA barriers and many problems per SM, larger problems more warps,
     // unless there are more problems than SMs and rounds are small (eps = 0.01,
-    // ms at 128 / 256 / 512 threads: 512 problems up to 300 rows 0.95 / 1.15 /
-    // 1.44; 300 up to 700: 1.03 / 0.73 / 1.09; 100 up to 1024: 0.93 / 0.64 / 0.59;
-    // 512 up to 2048: 2.37 / 2.00 / 2.32; at eps = 0.1, 300 up to 1500: 1.27 /
-    // 0.87 / 0.66).  The order of the cost sum stays that of kCostSums partial
+    // ms at 128 / 256 / 512 threads: 512 problems up to 300 rows 1.10 / 1.22 /
+    // 1.46; 300 up to 700: 0.90 / 0.64 / 0.99; 100 up to 1024: 0.98 / 0.73 / 0.77;
+    // 512 up to 2048: 2.26 / 1.93 / 2.19; at eps = 0.1, 300 up to 1500: 1.36 /
+    // 0.90 / 0.66).  The order of the cost sum stays that of kCostSums partial
     // sums.
     const DeviceInfo &di = device_info();
     const bool many = P > di.sms && floor(1.0 / eps) > 20.0;

@@ -55,12 +55,12 @@ inline bool solo_fits(int n_rows, int n_cols, int row_bytes, long long K) {
 
 // At floor(1/eps) <= kNearMaxK most of a solve can be one phase of a hundred
 // rounds in which hundreds of rows lose the same columns (squared distances, n
-// = 1000, eps = 0.1: 131 rounds of 464 rows).  The grid's rounds cost 4.3 us,
-// one CTA's 2.3 us at 512 to 1024 rows, so one CTA takes over inside a phase
-// that has lasted kMidRounds rounds: that solve 574 -> 347 us, n = 1500 855 -> 552
-// us, n = 1000 at eps = 0.3 1545 -> 701 us.  (A problem of 20 rounds is faster on
-// the grid: n = 1000, Euclidean, 122 us against 153 us on one CTA; at n = 2000
-// such a problem is 8 % slower with the take-over, 228 against 210 us.)
+// = 1000, eps = 0.1: 131 rounds of 464 rows).  The grid's rounds cost 4 us, one
+// CTA's 2 us at 512 to 1024 rows, so one CTA takes over inside a phase that has
+// lasted kMidRounds rounds: that solve 534 -> 320 us, n = 1500 835 -> 547 us,
+// Euclidean costs, eps = 0.3 497 -> 300 us.  (Problems of 20 to 30 rounds gain
+// little: Euclidean, eps = 0.1, grid / take-over / one CTA n = 1000 119 / 109 / 118
+// us, n = 1536 164 / 155 / 215.)
 constexpr int kMidRows = 1536;
 
 // Whether one CTA runs the problem from the start (solo), takes over from the

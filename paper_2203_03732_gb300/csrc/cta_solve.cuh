@@ -24,9 +24,9 @@
 //     barrier (KEEP: one problem alone; with several problems per SM their
 //     other warps hide that latency, and it measured 3 % slower).
 //
-// The 512-problem batch (64 to 2048 rows, eps = 0.01) took 2.60 ms in the
+// The 512-problem batch (64 to 2048 rows, eps = 0.01) took 2.59 ms in the
 // solver with 64-bit words, past-proposal lists and a word lookup per taken
-// candidate; it takes 1.52 ms.  64 problems of 4096 points: 7.0 ms -> 1.2 ms.
+// candidate; it takes 1.23 ms.  64 problems of 4096 points: 7.0 ms -> 1.19 ms.
 // A round of few rows (n = 1000) takes about 1.5 us, of which the scan of a
 // row is 0.9 us: instructions of one warp, not its loads.  Measured and left
 // out: 4 or 8 lanes per row (the lanes' shared-memory and L1 accesses cost
@@ -593,7 +593,7 @@ __device__ __forceinline__ int cta_scan_excl(int flag, CtaShared &s) {
 // After cta_phases: matching out of the words, completion (the k-th free row
 // takes the k-th free column, Sec. 2.1), duals and the FP64 cost, each to
 // global memory.  The cost is summed as `sums` strided partial sums (a power
-// of two, at least blockDim.x) and a halving tree over them, in `part`
+// of two; threads past it idle) and a halving tree over them, in `part`
 // (shared memory, `sums` doubles), so its order depends on `sums` alone.
 template <class CB, class Cost>
 __device__ __forceinline__ void cta_finish(CtaShared &s, unsigned char *dyn, const CtaLayout &L, int nB, int nA,
