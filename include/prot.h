@@ -287,7 +287,7 @@ pr_status pr_assign_batched(const void *C, pr_dtype dt, int32_t n_problems, cons
  * the matched distance sum in input units, evaluated in FP64.  Coordinates
  * that make a distance of any problem non-finite give PR_ERR_INVALID (reported
  * when the call synchronises).  After an error the problems that were not
- * solved have cost NaN, and pr_assign_backward gives NaN on their rows.
+ * solved have cost NaN and the identity as their matching.
  */
 pr_status pr_assign_batched_points(const float *XA, const float *XB, int32_t dim, pr_metric metric,
                                    int32_t n_problems, const int32_t *n_host, double eps,
@@ -409,9 +409,7 @@ pr_status pr_ot(const void *C, pr_dtype dt, int64_t ldc, int32_t n_sup, int32_t 
  *   grad_Y     [batch][n][dim] out: minus that, at row sigma(i)
  *   grad_C     [batch][n][n] out or NULL: g / n on matched entries, else 0
  * Each value is formed in FP64 as ((x - y) * 2) / n * g and rounded once.
- * Asynchronous; the plans must be permutations (not checked on the device),
- * except that a problem which pr_assign_batched_points left unsolved after an
- * error may be passed on: its gradients are NaN.
+ * Asynchronous; the plans must be permutations (not checked on the device).
  */
 pr_status pr_assign_backward(const int32_t *row_to_col, const float *X, const float *Y,
                              int32_t batch, int32_t n, int32_t dim, const float *grad_cost,

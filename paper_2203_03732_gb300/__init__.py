@@ -539,6 +539,7 @@ def _assign_loss_function():
         @staticmethod
         def backward(ctx, g):
             X, Y, r2c = ctx.saved_tensors
+            g = g.add(ctx.plan["costs"], alpha=0)  # NaN where the pair was not solved
             gX, gY = assign_backward(r2c, X.detach(), Y.detach(), g)
             return gX, gY, None
 

@@ -28,10 +28,6 @@ __global__ void k_backward(const int32_t *__restrict__ r2c, const float *__restr
          t += (long long)gridDim.x * blockDim.x) {
         const int p = (int)(t / n);
         const int j = r2c[t];
-        if (j == kUnsolved) {  // no plan, on any row of the pair: NaN
-            for (int k = 0; k < dim; ++k) gX[t * dim + k] = gY[t * dim + k] = __int_as_float(0x7FC00000);
-            continue;
-        }
         if (j < 0 || j >= n) continue;  // not a completed plan: entries left unwritten
         const double gp = (double)g[p];
         const float *x = X + t * dim;
@@ -55,9 +51,7 @@ __global__ void k_grad_c(const int32_t *__restrict__ r2c, int batch, int n,
         const long long pi = t / n;  // pair * n + row
         const int j = (int)(t - pi * n);
         const int p = (int)(pi / n);
-        gC[t] = r2c[pi] == j           ? __double2float_rn(__ddiv_rn((double)g[p], (double)n))
-                : r2c[pi] == kUnsolved ? __int_as_float(0x7FC00000)
-                                       : 0.0f;
+        gC[t] = r2c[pi] == j ? __double2float_rn(__ddiv_rn((double)g[p], (double)n)) : 0.0f;
     }
 }
 

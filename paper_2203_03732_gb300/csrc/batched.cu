@@ -303,11 +303,13 @@ struct BatchCost {
     }
 };
 
-// Outputs of a problem that is not solved, because an error was recorded (an
-// asynchronous loss and its gradients are then NaN, not what the buffers held).
+// Outputs of a problem that is not solved, because an error was recorded: cost
+// NaN, and mates that are indices all the same (the identity), so that an
+// asynchronous caller neither takes what the buffers held for a result nor
+// reads out of range with it.
 __device__ void write_unsolved(const BParams &p, const BDesc &D, int pi) {
     for (int i = threadIdx.x; i < D.n; i += blockDim.x) {
-        p.row_to_col[D.v_off + i] = p.col_to_row[D.v_off + i] = kUnsolved;
+        p.row_to_col[D.v_off + i] = p.col_to_row[D.v_off + i] = i;
         p.y_row[D.v_off + i] = p.y_col[D.v_off + i] = 0;
     }
     if (threadIdx.x == 0) {

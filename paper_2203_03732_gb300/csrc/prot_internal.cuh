@@ -63,9 +63,6 @@ struct WsHead {
 };
 constexpr int kWsMagic = 0x70725f31;  // "pr_1"
 
-// row_to_col of a batched problem that was not solved (an error was recorded).
-constexpr int kUnsolved = INT32_MIN;
-
 // ---------------------------------------------------------------------------
 // Device memory-order primitives (gpu scope)
 // ---------------------------------------------------------------------------

@@ -65,3 +65,16 @@ def test_loss_and_gradients_are_nan(prot, tmp_path, monkeypatch, dim):
     loss = prot.assignment_loss(X, Y, 0.1)
     gX, gY = torch.autograd.grad(loss.sum(), (X, Y))
     assert torch.isnan(loss).all() and torch.isnan(gX).all() and torch.isnan(gY).all()
+
+
+def test_unsolved_problems_have_indices_in_range(prot):
+    """After an error an asynchronous caller may still index with the mates."""
+    import torch
+    XA, XB = (torch.from_numpy(x).cuda() for x in clouds(3, "one nan"))
+    got = prot.assign_batched_points(XA, XB, SIZES, 0.1, sync=False)
+    off = 0
+    for n in SIZES:
+        want = torch.arange(int(n), dtype=torch.int32, device="cuda")
+        for k in ("row_to_col", "col_to_row"):
+            assert torch.equal(got[k][off:off + int(n)], want), k
+        off += int(n)
