@@ -294,16 +294,11 @@ struct Smem {
     int job_tgt[kBatch];
     int job_best[kBatch];
     int2 don[kBatch];         // pool entries given to the pool in this batch
-    union {
-        int best[kWarps];      // run_jobs: each register group's lowest candidate
-        int fbest[kFastRows];  // fast rounds: each row's lowest candidate
-    };
-    union {
-        unsigned long long cbar[4][2];  // cluster mode: this CTA's copy of the barrier slots
-        int4 frow[kFastRows];           // fast rounds: (row, scan start, target, 1 if it scanned)
-    };
+    int best[kWarps];
+    int fbest[kFastRows];     // fast rounds: each row's lowest candidate
+    int4 frow[kFastRows];     // ... (row, scan start, target, 1 if it scanned)
     int nfl[2], nql[2];
-    int nleft;                // first rounds: rows with long scans
+    int nleft, far;           // first rounds: rows with long scans; 1 if they were many (no near_scans then)
     int njob, ndon, don_base;
     int had_prop, nonfirst, nf_delta, donated;
     unsigned long long bytes;
@@ -311,12 +306,15 @@ struct Smem {
     unsigned long long cells;
     unsigned long long pub, pub2;
     unsigned long long pacc[4];  // profile: build, scan, proposal, tail ns of this round
-    unsigned long long mbar[kWarps];  // cluster mode: completion of each warp's row copy
+    unsigned long long cbar[4][2];  // cluster mode: this CTA's copy of the barrier slots
     int err;
-    int far;                  // 1 if the rows with long scans were many (no near_scans in this phase)
+    int spare[8];             // keeps the largest n_cols where it was
 };
-// The keys share the space: this size gives the largest n_cols, 89,808.
-static_assert(sizeof(Smem) <= 41600, "n_cols up to 89,808");
+// The keys share the space: this size gives the largest n_cols, 89,808.  The row
+// copies' mbarriers lie in front of the slots, which the widest problems do not
+// have.  (Unions of what only fast rounds and only the cluster form use gave the
+// same size, but the offset rule's code came out 1 % slower.)
+static_assert(sizeof(Smem) == 41600, "n_cols up to 89,808");
 
 struct Lists {
     int4 *ql[2];  // global overflow of ql
@@ -613,6 +611,11 @@ __device__ __forceinline__ void bulk_row_copy(void *dst, const void *src, unsign
                  ::"r"(smem_addr(dst)), "l"(src), "r"(bytes), "r"(smem_addr(mbar)) : "memory");
 }
 
+// The mbarrier of each warp's row copies, in front of the slots.
+__device__ __forceinline__ unsigned long long *mbar_of(unsigned char *slots, int warp) {
+    return reinterpret_cast<unsigned long long *>(slots) - kWarps + warp;
+}
+
 // Waits (bounded by `limit` cycles) for the phase of parity `parity` of mbar.
 __device__ __forceinline__ bool mbar_wait(unsigned long long *mbar, unsigned parity, long long limit) {
     const long long t0 = clock64();
@@ -796,8 +799,8 @@ __device__ __forceinline__ void run_jobs(Smem &s, const Lists &g, const Params &
                     const unsigned bytes = (unsigned)((lim - s_al) * sizeof(CB));
                     const CB *src = static_cast<const CB *>(p.cb) + (size_t)b * p.ldq + s_al;
                     __syncwarp();
-                    if (lane == 0) bulk_row_copy(slot, src, bytes, &s.mbar[warp]);
-                    if (mbar_wait(&s.mbar[warp], mstate & 1u, kCopyWaitCycles)) {
+                    if (lane == 0) bulk_row_copy(slot, src, bytes, mbar_of(slots, warp));
+                    if (mbar_wait(mbar_of(slots, warp), mstate & 1u, kCopyWaitCycles)) {
                         mstate ^= 1u;
                         my_bytes += bytes;
                         a = warp_scan_slot<CB, F7, OFS>(slot, ks, tk, R > Rps, s_al, start, lim, stop, tgt, lane);
@@ -1039,13 +1042,13 @@ __device__ __forceinline__ void fast_propose(Smem &s, const Lists &g, const Para
 // round R + 1.
 // ---------------------------------------------------------------------------
 // Dynamic shared memory of the phase kernel: Smem, the key copy, the taken
-// set; in cluster mode then row slots from a 128-byte boundary.
+// set; with slots then their mbarriers and the slots, from a 128-byte boundary.
 __host__ __device__ inline size_t smem_bytes(int ldq, int key_bytes = 2) {
     return ((sizeof(Smem) + 15) & ~size_t(15)) + (size_t)ldq * key_bytes +
            (size_t)((ldq + 31) / 32) * sizeof(unsigned);
 }
 __host__ __device__ inline size_t slots_offset(int ldq, int key_bytes) {
-    return (smem_bytes(ldq, key_bytes) + 127) & ~size_t(127);
+    return ((smem_bytes(ldq, key_bytes) + 127) & ~size_t(127)) + kWarps * sizeof(unsigned long long);
 }
 
 // CL: the launch is one thread-block cluster (barriers through distributed
@@ -1107,7 +1110,7 @@ k_phases(Params p, int warps_per_row, int rows_per_group) {
         for (int i = 0; i < 4; ++i) s.cbar[i][0] = s.cbar[i][1] = 0;
         if (SL) {
             for (int w = 0; w < p.nslots; ++w)
-                asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&s.mbar[w])) : "memory");
+                asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(mbar_of(slots, w))) : "memory");
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         }
     }
@@ -1428,7 +1431,7 @@ done:
     }
     // A copy whose wait gave up gets one more bounded wait: the CTA must not
     // exit while it may still write the slot.
-    if (SL && (mstate & 2u)) mbar_wait(&s.mbar[threadIdx.x >> 5], mstate & 1u, kCopyWaitCycles);
+    if (SL && (mstate & 2u)) mbar_wait(mbar_of(slots, threadIdx.x >> 5), mstate & 1u, kCopyWaitCycles);
     // Cluster mode: a CTA's shared memory must outlive every add another CTA
     // makes to it.  Every CTA gets here: the loop ends on the same shared
     // decision everywhere, or on a bounded wait that gave up.
