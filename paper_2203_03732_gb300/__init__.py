@@ -534,12 +534,13 @@ def _assign_loss_function():
                                         sizes, eps, metric="sqeuclidean", sync=False, tune="auto")
             ctx.save_for_backward(X, Y, res["row_to_col"])
             ctx.plan = res
-            return (res["costs"] / n).to(X.dtype)
+            return torch.div(res["costs"], n, out=torch.empty(B, dtype=X.dtype, device=X.device))
 
         @staticmethod
         def backward(ctx, g):
             X, Y, r2c = ctx.saved_tensors
-            g = g.add(ctx.plan["costs"], alpha=0)  # NaN where the pair was not solved
+            # NaN where the pair was not solved (one operation, in g's type)
+            g = torch.add(g.detach(), ctx.plan["costs"], alpha=0, out=torch.empty(g.shape, dtype=g.dtype, device=g.device))
             gX, gY = assign_backward(r2c, X.detach(), Y.detach(), g)
             return gX, gY, None
 
